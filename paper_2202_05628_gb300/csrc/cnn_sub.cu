@@ -66,20 +66,20 @@ __host__ __device__ constexpr int skip_min(int v) { return v == 2 ? 1 : 0; }
 // (ox = -1, 0) and px = 1 (ox = 0, 1).
 __host__ __device__ constexpr int up_n(int v) { return v == 0 ? 2 : 1; }
 __host__ __device__ constexpr int up_min(int v) { return v == 1 ? 1 : 0; }
-// First weight block of (r, c) among row phase py's skip entries, ordered by
-// r (py - 1 .. py + 1), c, then px; of (oy, ox) among its low-resolution
-// entries, ordered by oy (py - 1, py), ox, then px.
-__host__ __device__ constexpr int skip_base(int py, int r, int c) {
-  int b = 6 * (r - (py - 1));
+// First weight block of column offset c among one input row's six skip
+// entries (ordered by c, then px; the rows r = py - 1 .. py + 1 follow each
+// other), of ox among one low-resolution row's four (rows oy = py - 1, py).
+__host__ __device__ constexpr int skip_block(int c) {
+  int b = 0;
   for (int cc = -1; cc < c; ++cc) b += skip_n(cc);
   return b;
 }
-__host__ __device__ constexpr int up_base(int py, int oy, int ox) {
-  int b = 4 * (oy - (py - 1));
+__host__ __device__ constexpr int up_block(int ox) {
+  int b = 0;
   for (int xx = -1; xx < ox; ++xx) b += up_n(xx);
   return b;
 }
-static_assert(skip_base(0, 1, 2) + 1 == kSkipEntries && up_base(1, 1, 1) + 1 == kUpEntries, "entry tables");
+static_assert(3 * (skip_block(2) + 1) == kSkipEntries && 2 * (up_block(1) + 1) == kUpEntries, "entry tables");
 
 // floor(v / 2) for v in {-1, 0, 1, 2}
 __host__ __device__ constexpr int half_floor(int v) { return (v + 2) / 2 - 1; }
@@ -129,8 +129,6 @@ __global__ void __launch_bounds__(kThreads, kCtas)
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int py = blockIdx.x & 1;                  // this CTA's output rows 2i + py
   const int u0 = blockIdx.x >> 1, du = gridDim.x >> 1;
-  const int n_skip = 6 * p.cs_ch;                 // skip stages: per chunk 3 rows x (even, odd) boxes
-  const int n_stage_unit = n_skip + 2 * p.cu_ch;  // + per chunk 2 low-resolution rows
   const int ubase_off = p.cs_ch * kSkipEntries * kBlock;
 
   if (threadIdx.x == 0) {
@@ -171,24 +169,40 @@ __global__ void __launch_bounds__(kThreads, kCtas)
     if (lane == 0) {
       int s = 0;
       uint32_t ph = 0;
-      for (int u = u0; u < p.n_units && !*abort_flag; u += du) {
-        const int i = u / p.tiles_per_row, j0 = (u % p.tiles_per_row) * 128;
-        for (int st = 0; st < n_stage_unit; ++st) {
-          if (!mbar_wait(&empty[s], ph ^ 1u, abort_flag)) break;
-          uint8_t* dst = stages + (size_t)s * kStageBytes;
-          mbar_expect_tx(&full[s], (uint32_t)kBoxBytes);
-          if (st < n_skip) {
-            const int cc = st / 6, k = st - 6 * cc, r = py - 1 + (k >> 1), q = k & 1;
-            tma_load_4d(dst, &tmS, &full[s], cc * kKC, j0 - 1, q, 2 * i + r);
-          } else {
-            const int t = st - n_skip, cc = t >> 1, oy = py - 1 + (t & 1);
-            tma_load_3d(dst, &tmU, &full[s], cc * kKC, j0 - 1, i + oy);
-          }
-          if (++s == S) {
-            s = 0;
-            ph ^= 1u;
-          }
+      bool ok = true;
+      // the next free stage, announced to its barrier (null: aborted)
+      auto acquire = [&]() -> uint8_t* {
+        if (!mbar_wait(&empty[s], ph ^ 1u, abort_flag)) {
+          ok = false;
+          return nullptr;
         }
+        mbar_expect_tx(&full[s], (uint32_t)kBoxBytes);
+        return stages + (size_t)s * kStageBytes;
+      };
+      auto advance = [&]() {
+        if (++s == S) {
+          s = 0;
+          ph ^= 1u;
+        }
+      };
+      for (int u = u0; ok && u < p.n_units && !*abort_flag; u += du) {
+        const int i = u / p.tiles_per_row, j0 = (u - i * p.tiles_per_row) * 128;
+        // the boxes in order by nested loops (no divisions on the issuing thread)
+        for (int cc = 0; cc < p.cs_ch; ++cc)
+          for (int r = py - 1; r <= py + 1; ++r)
+            for (int q = 0; ok && q < 2; ++q) {
+              uint8_t* dst = acquire();
+              if (!dst) break;
+              tma_load_4d(dst, &tmS, &full[s], cc * kKC, j0 - 1, q, 2 * i + r);
+              advance();
+            }
+        for (int cc = 0; cc < p.cu_ch; ++cc)
+          for (int oy = py - 1; ok && oy <= py; ++oy) {
+            uint8_t* dst = acquire();
+            if (!dst) break;
+            tma_load_3d(dst, &tmU, &full[s], cc * kKC, j0 - 1, i + oy);
+            advance();
+          }
       }
     }
   } else if (warp == 1) {
@@ -199,41 +213,44 @@ __global__ void __launch_bounds__(kThreads, kCtas)
       uint32_t ph = 0, aph = 0;
       bool ok = mbar_wait(wbar, 0u, abort_flag);
       const uint32_t wbase = smem_u32(wsm), ubase = wbase + (uint32_t)ubase_off;
+      uint32_t a0 = 0;  // the stage in hand
+      auto next_full = [&]() {
+        if (!mbar_wait(&full[s], ph, abort_flag)) return false;
+        tc_fence_after();
+        a0 = smem_u32(stages + (size_t)s * kStageBytes);
+        return true;
+      };
+      auto release = [&]() {
+        umma_commit(&empty[s]);
+        if (++s == S) {
+          s = 0;
+          ph ^= 1u;
+        }
+      };
       for (int u = u0; ok && u < p.n_units && !*abort_flag; u += du) {
         // the epilogue clears the accumulators (phase 0 = the initial clear)
         if (!mbar_wait(&acce[buf], aph, abort_flag)) break;
         tc_fence_after();
         const uint32_t d0 = tmem_base + (uint32_t)(buf * kAccCols);
-        for (int st = 0; st < n_stage_unit; ++st) {
-          if (!mbar_wait(&full[s], ph, abort_flag)) {
-            ok = false;
-            break;
-          }
-          tc_fence_after();
-          const uint32_t a0 = smem_u32(stages + (size_t)s * kStageBytes);
-          if (st < n_skip) {
-            const int cc = st / 6, k = st - 6 * cc, r = py - 1 + (k >> 1), q = k & 1;
-            // even box: c = 0 (from row 1), c = 2 (row 2); odd box: c = -1 (row 0), c = 1 (row 1)
+        uint32_t wb = wbase;  // weight blocks of the (chunk, row) in hand
+        // even box: c = 0 (from row 1), c = 2 (row 2); odd box: c = -1 (row 0), c = 1 (row 1)
+        for (int cr = 0; ok && cr < 3 * p.cs_ch; ++cr, wb += 6 * kBlock) {
+          if (!(ok = next_full())) break;
+          sub_mma(d0, a0 + 1 * kKCB, wb + skip_block(0) * kBlock, skip_n(0), skip_min(0));
+          sub_mma(d0, a0 + 2 * kKCB, wb + skip_block(2) * kBlock, skip_n(2), skip_min(2));
+          release();
+          if (!(ok = next_full())) break;
+          sub_mma(d0, a0 + 0 * kKCB, wb + skip_block(-1) * kBlock, skip_n(-1), skip_min(-1));
+          sub_mma(d0, a0 + 1 * kKCB, wb + skip_block(1) * kBlock, skip_n(1), skip_min(1));
+          release();
+        }
+        wb = ubase;
+        for (int co = 0; ok && co < 2 * p.cu_ch; ++co, wb += 4 * kBlock) {
+          if (!(ok = next_full())) break;
 #pragma unroll
-            for (int t = 0; t < 2; ++t) {
-              const int c = q == 0 ? 2 * t : 2 * t - 1;
-              const int off = q == 0 ? t + 1 : t;
-              const uint32_t wb0 = wbase + (uint32_t)((cc * kSkipEntries + skip_base(py, r, c)) * kBlock);
-              sub_mma(d0, a0 + (uint32_t)(off * kKCB), wb0, skip_n(c), skip_min(c));
-            }
-          } else {
-            const int t = st - n_skip, cc = t >> 1, oy = py - 1 + (t & 1);
-#pragma unroll
-            for (int ox = -1; ox <= 1; ++ox) {
-              const uint32_t wb0 = ubase + (uint32_t)((cc * kUpEntries + up_base(py, oy, ox)) * kBlock);
-              sub_mma(d0, a0 + (uint32_t)((ox + 1) * kKCB), wb0, up_n(ox), up_min(ox));
-            }
-          }
-          umma_commit(&empty[s]);
-          if (++s == S) {
-            s = 0;
-            ph ^= 1u;
-          }
+          for (int ox = -1; ox <= 1; ++ox)
+            sub_mma(d0, a0 + (uint32_t)((ox + 1) * kKCB), wb + up_block(ox) * kBlock, up_n(ox), up_min(ox));
+          release();
         }
         if (!ok) break;
         umma_commit(&accf[buf]);

@@ -430,8 +430,7 @@ __global__ void __launch_bounds__(kThreads, TcCfg<N, KCB, F8>::kCtas)
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int cpt = p.cin / KC;  // K chunks per tap
-  const int n_skip = 9 * p.cs_ch;  // sub-pixel tiles: the skip part's chunks, then 4 taps x cu_ch
-  const int n_chunks = p.sub ? n_skip + 4 * p.cu_ch : 9 * cpt;
+  const int n_chunks = p.sub ? 9 * p.cs_ch + 4 * p.cu_ch : 9 * cpt;  // (sub-pixel tiles: the skip part's, then 4 taps x cu_ch)
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < Cfg::kStages; ++s) {
@@ -469,36 +468,63 @@ __global__ void __launch_bounds__(kThreads, TcCfg<N, KCB, F8>::kCtas)
     if (lane == 0) {
       int s = 0;
       uint32_t ph = 0;
-      for (int tile = blockIdx.x; tile < p.n_tiles && !*abort_flag; tile += gridDim.x) {
+      bool ok = true;
+      // the next free stage, announced to its barrier (null: aborted)
+      auto acquire = [&]() -> uint8_t* {
+        if (!mbar_wait(&empty[s], ph ^ 1u, abort_flag)) {
+          ok = false;
+          return nullptr;
+        }
+        mbar_expect_tx(&full[s], Cfg::kStage);
+        return stages + s * Cfg::kStage;
+      };
+      auto advance = [&]() {
+        if (++s == Cfg::kStages) {
+          s = 0;
+          ph ^= 1u;
+        }
+      };
+      // the K chunks in order by nested loops: a stage costs the issuing thread
+      // ~250 cycles (wait, expect, TMA) and cost it ~480 with the divisions that
+      // named its tap and chunk (1920x1080 BF16 network 766 -> 718 us with this in
+      // all three convolution kernels)
+      for (int tile = blockIdx.x; ok && tile < p.n_tiles && !*abort_flag; tile += gridDim.x) {
         const int st = p.sub ? tile >> 2 : tile, oph = tile & 3;  // (sub-pixel: output phase (py, px))
-        const int y = st / p.tiles_per_row, x0 = (st % p.tiles_per_row) * 128;
-        for (int c = 0; c < n_chunks; ++c) {
-          if (!mbar_wait(&empty[s], ph ^ 1u, abort_flag)) break;
-          uint8_t* a = stages + s * Cfg::kStage;
-          mbar_expect_tx(&full[s], Cfg::kStage);
-          if (!p.sub) {
-            const int tap = c / cpt, cc = c - tap * cpt;
-            const int r = tap / 3, q = tap - 3 * (tap / 3);
-            tma_load_3d(a, &tmA, &full[s], cc * KC, x0 + q - 1, y + r - 1);
-            tma_load_2d(a + Cfg::kA, &tmB, &full[s], tap * p.cin + cc * KC, 0);
-          } else if (c < n_skip) {
-            // skip tap (dy, dx): input column 2x + px + dx = 2 (x + jo) + q of the x-phase split rows
-            const int tap = c / p.cs_ch, cc = c - tap * p.cs_ch;
-            const int dy = tap / 3 - 1, cpos = (oph & 1) + tap % 3 - 1;
-            const int q = cpos & 1, jo = (cpos - q) / 2;
-            tma_load_4d(a, &tmA, &full[s], cc * KC, x0 + jo, q, 2 * y + (oph >> 1) + dy);
-            tma_load_2d(a + Cfg::kA, &tmB, &full[s], tap * p.cs_ch * KC + cc * KC, oph * N);
-          } else {
-            // low-resolution tap (oy, ox), oy in {py - 1, py}, ox in {px - 1, px}
-            const int t = c - n_skip, tu = t / p.cu_ch, cc = t - tu * p.cu_ch;
-            const int oy = (oph >> 1) - 1 + (tu >> 1), ox = (oph & 1) - 1 + (tu & 1);
-            tma_load_3d(a, &tmU, &full[s], cc * KC, x0 + ox, y + oy);
-            tma_load_2d(a + Cfg::kA, &tmB, &full[s], (9 * p.cs_ch + tu * p.cu_ch) * KC + cc * KC, oph * N);
-          }
-          if (++s == Cfg::kStages) {
-            s = 0;
-            ph ^= 1u;
-          }
+        const int y = st / p.tiles_per_row, x0 = (st - y * p.tiles_per_row) * 128;
+        int k = 0;  // first weight column of the chunk
+        if (!p.sub) {
+          for (int r = -1; r <= 1; ++r)
+            for (int q = -1; q <= 1; ++q)
+              for (int cc = 0; ok && cc < cpt; ++cc, k += KC) {
+                uint8_t* a = acquire();
+                if (!a) break;
+                tma_load_3d(a, &tmA, &full[s], cc * KC, x0 + q, y + r);
+                tma_load_2d(a + Cfg::kA, &tmB, &full[s], k, 0);
+                advance();
+              }
+        } else {
+          // skip taps (dy, dx): input column 2x + px + dx = 2 (x + jo) + q of the x-phase split rows
+          for (int dy = -1; dy <= 1; ++dy)
+            for (int dx = -1; dx <= 1; ++dx) {
+              const int cpos = (oph & 1) + dx, q = cpos & 1, jo = (cpos - q) / 2;
+              for (int cc = 0; ok && cc < p.cs_ch; ++cc, k += KC) {
+                uint8_t* a = acquire();
+                if (!a) break;
+                tma_load_4d(a, &tmA, &full[s], cc * KC, x0 + jo, q, 2 * y + (oph >> 1) + dy);
+                tma_load_2d(a + Cfg::kA, &tmB, &full[s], k, oph * N);
+                advance();
+              }
+            }
+          // low-resolution taps (oy, ox), oy in {py - 1, py}, ox in {px - 1, px}
+          for (int oy = (oph >> 1) - 1; oy <= (oph >> 1); ++oy)
+            for (int ox = (oph & 1) - 1; ox <= (oph & 1); ++ox)
+              for (int cc = 0; ok && cc < p.cu_ch; ++cc, k += KC) {
+                uint8_t* a = acquire();
+                if (!a) break;
+                tma_load_3d(a, &tmU, &full[s], cc * KC, x0 + ox, y + oy);
+                tma_load_2d(a + Cfg::kA, &tmB, &full[s], k, oph * N);
+                advance();
+              }
         }
       }
     }
@@ -599,13 +625,10 @@ struct RowCfg {
   static constexpr int kSlots = kRows;
   static constexpr int kBufCols = kSlots * N;  // columns of one accumulator buffer
   static constexpr int kHalo = 130;                                   // input pixels of a row box (128 + 2)
-  // input rows per stage (one box); two measured slower on the 32-channel
-  // layers (a deeper box per barrier round trip, half as many stages in flight)
-  static constexpr int kStageRows = 1;
-  static constexpr int kRowBytes = kHalo * KCB;                       // one input row of the box
-  static constexpr int kBoxBytes = kStageRows * kRowBytes;
+  // one input row per stage; two measured slower on the 32-channel layers
+  // (a deeper box per barrier round trip, half as many stages in flight)
+  static constexpr int kBoxBytes = kHalo * KCB;
   static constexpr int kStageBytes = (kBoxBytes + 1023) / 1024 * 1024;  // stages stay on swizzle-atom boundaries
-  static_assert((kRows + 2) % kStageRows == 0, "a unit's input rows fill whole stages");
 };
 
 struct RowParams {
@@ -643,8 +666,7 @@ __global__ void __launch_bounds__(kThreads, 2)
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int cpt = rp.cpt;
-  const int n_stage_unit = (kRows + 2) / Cfg::kStageRows * cpt;  // stages per unit
-  const int kStage = Cfg::kStageBytes;  // one box of kStageRows rows of 130 pixels: the three shifts are row offsets
+  const int kStage = Cfg::kStageBytes;  // one box of 130 pixels of a row: the three shifts are row offsets
   // the swizzle follows the absolute shared-memory address, so a descriptor
   // may start at any row of the box: shift dx is the box from row dx on
   // resident weight block of (dy + 1, dx + 1, chunk): the three vertical
@@ -679,8 +701,8 @@ __global__ void __launch_bounds__(kThreads, 2)
   const uint32_t tmem_base = *tmem_slot;
   float amax = 0.0f;
 
-  // A stage is kStageRows input rows of one channel chunk (one box, one
-  // barrier round trip); each row serves the three horizontal shifts.
+  // A stage is one input row of one channel chunk (one box, one barrier
+  // round trip); it serves the three horizontal shifts.
   grid_dep_launch();  // the next layer may start its prologue where this one's CTAs leave SMs
   if (warp == 0) {
     // ------------------------------------------------------------ TMA
@@ -694,19 +716,22 @@ __global__ void __launch_bounds__(kThreads, 2)
     if (lane == 0) {
       int s = 0;
       uint32_t ph = 0;
-      for (int u = blockIdx.x; u < rp.n_units && !*abort_flag; u += gridDim.x) {
-        const int y0 = (u / p.tiles_per_row) * kRows, x0 = (u % p.tiles_per_row) * 128;
-        for (int st = 0; st < n_stage_unit; ++st) {
-          if (!mbar_wait(&empty[s], ph ^ 1u, abort_flag)) break;
-          const int jj = st / cpt, c = st - jj * cpt;
-          uint8_t* dst = stages + (size_t)s * kStage;
-          mbar_expect_tx(&full[s], (uint32_t)Cfg::kBoxBytes);
-          tma_load_3d(dst, &tmA, &full[s], c * Cfg::KC, x0 - 1, y0 - 1 + jj * Cfg::kStageRows);
-          if (++s == S) {
-            s = 0;
-            ph ^= 1u;
+      bool ok = true;
+      for (int u = blockIdx.x; ok && u < rp.n_units && !*abort_flag; u += gridDim.x) {
+        const int uy = u / p.tiles_per_row, y0 = uy * kRows, x0 = (u - uy * p.tiles_per_row) * 128;
+        for (int j = 0; ok && j < kRows + 2; ++j)
+          for (int c = 0; c < cpt; ++c) {
+            if (!mbar_wait(&empty[s], ph ^ 1u, abort_flag)) {
+              ok = false;
+              break;
+            }
+            mbar_expect_tx(&full[s], (uint32_t)Cfg::kBoxBytes);
+            tma_load_3d(stages + (size_t)s * kStage, &tmA, &full[s], c * Cfg::KC, x0 - 1, y0 - 1 + j);
+            if (++s == S) {
+              s = 0;
+              ph ^= 1u;
+            }
           }
-        }
       }
     }
   } else if (warp == 1) {
@@ -722,22 +747,19 @@ __global__ void __launch_bounds__(kThreads, 2)
         if (!mbar_wait(&acce[buf], aph, abort_flag)) break;
         tc_fence_after();
         const uint32_t d0 = tmem_base + (uint32_t)(buf * Cfg::kBufCols);
-        for (int st = 0; st < n_stage_unit; ++st) {
-          if (!mbar_wait(&full[s], ph, abort_flag)) {
-            ok = false;
-            break;
-          }
-          tc_fence_after();
-          const int jj = st / cpt, c = st - jj * cpt;
-#pragma unroll
-          for (int r = 0; r < Cfg::kStageRows; ++r) {
-            const int j = jj * Cfg::kStageRows + r;
-            const uint32_t a0 = smem_u32(stages + (size_t)s * kStage) + (uint32_t)(r * Cfg::kRowBytes);
-            // input row j feeds output rows j - dyi of the unit for the taps dyi in [lo, hi]
-            // (slots R - 1 - j + lo ..., consecutive like the stacked taps' weight blocks)
-            const int lo = max(0, j - kRows + 1), hi = min(2, j);
-            const uint32_t dj = d0 + (uint32_t)((kRows - 1 - j + lo) * N);
-            const uint32_t idesc = F8 ? idesc_e4m3(128, (hi - lo + 1) * N) : idesc_bf16(128, (hi - lo + 1) * N);
+        for (int j = 0; ok && j < kRows + 2; ++j) {
+          // input row j feeds output rows j - dyi of the unit for the taps dyi in [lo, hi]
+          // (slots R - 1 - j + lo ..., consecutive like the stacked taps' weight blocks)
+          const int lo = max(0, j - kRows + 1), hi = min(2, j);
+          const uint32_t dj = d0 + (uint32_t)((kRows - 1 - j + lo) * N);
+          const uint32_t idesc = F8 ? idesc_e4m3(128, (hi - lo + 1) * N) : idesc_bf16(128, (hi - lo + 1) * N);
+          for (int c = 0; c < cpt; ++c) {
+            if (!mbar_wait(&full[s], ph, abort_flag)) {
+              ok = false;
+              break;
+            }
+            tc_fence_after();
+            const uint32_t a0 = smem_u32(stages + (size_t)s * kStage);
 #pragma unroll
             for (int dxi = 0; dxi < 3; ++dxi) {
               const uint32_t bw = wbase + (uint32_t)((wblk(0, dxi, c) + lo) * N * KCB);
@@ -745,11 +767,11 @@ __global__ void __launch_bounds__(kThreads, 2)
               for (int kk = 0; kk < KCB / 32; ++kk)
                 umma<F8>(dj, umma_desc<KCB>(a0 + dxi * KCB + kk * 32), umma_desc<KCB>(bw + kk * 32), idesc, 1u);
             }
-          }
-          umma_commit(&empty[s]);
-          if (++s == S) {
-            s = 0;
-            ph ^= 1u;
+            umma_commit(&empty[s]);
+            if (++s == S) {
+              s = 0;
+              ph ^= 1u;
+            }
           }
         }
         if (!ok) break;
@@ -1003,7 +1025,7 @@ art_status launch_rows(art_ctx* ctx, const TcConv& c) {
   {
     cuuint64_t dims[3] = {(cuuint64_t)c.cin, (cuuint64_t)c.W, (cuuint64_t)c.H};
     cuuint64_t strides[2] = {(cuuint64_t)c.cin * kEs, (cuuint64_t)c.W * c.cin * kEs};
-    cuuint32_t box[3] = {(cuuint32_t)Cfg::KC, (cuuint32_t)Cfg::kHalo, (cuuint32_t)Cfg::kStageRows};
+    cuuint32_t box[3] = {(cuuint32_t)Cfg::KC, (cuuint32_t)Cfg::kHalo, 1};
     cuuint32_t es[3] = {1, 1, 1};
     CUresult r = g_encode(&tmA, dt, 3, (void*)c.in, dims, strides, box, es,
                           CU_TENSOR_MAP_INTERLEAVE_NONE, swz, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
@@ -1060,7 +1082,7 @@ art_status launch_rows(art_ctx* ctx, const TcConv& c) {
   cudaFuncAttributes fa;
   const bool regs2 = cudaFuncGetAttributes(&fa, kfn) == cudaSuccess && 2 * kThreads * fa.numRegs <= 65536;
   // (at least three input rows in flight per CTA) and both CTAs' registers fit
-  const int ctas = (half >= (3 + Cfg::kStageRows - 1) / Cfg::kStageRows * Cfg::kStageBytes && regs2) ? 2 : 1;
+  const int ctas = (half >= 3 * Cfg::kStageBytes && regs2) ? 2 : 1;
   const int avail = 232448 / ctas - 1024 - rp.w_bytes - tail;
   rp.nbuf = (ctas == 2 && Cfg::kBufCols > 128) ? 1 : 2;  // 512 TMEM columns per SM
   rp.n_stages = std::min(24, avail / Cfg::kStageBytes);
