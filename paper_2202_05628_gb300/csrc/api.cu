@@ -195,6 +195,8 @@ void free_all(art_ctx* ctx) {
     if (L.wbf) cudaFree(L.wbf);
     if (L.wsub) cudaFree(L.wsub);
     if (L.wtap) cudaFree(L.wtap);
+    if (L.wx) cudaFree(L.wx);
+    if (L.wxu) cudaFree(L.wxu);
     if (L.w8) cudaFree(L.w8);
     if (L.wscale) cudaFree(L.wscale);
   }
@@ -911,6 +913,8 @@ art_status art_load_shader(art_ctx* ctx, const art_net_desc* desc, const float* 
     if (L.wbf) cudaFree(L.wbf);
     if (L.wsub) cudaFree(L.wsub);
     if (L.wtap) cudaFree(L.wtap);
+    if (L.wx) cudaFree(L.wx);
+    if (L.wxu) cudaFree(L.wxu);
     if (L.w8) cudaFree(L.w8);
     if (L.wscale) cudaFree(L.wscale);
   }
@@ -976,6 +980,41 @@ art_status art_load_shader(art_ctx* ctx, const art_net_desc* desc, const float* 
     if (st == ART_OK) st = tap_blocks(10, d.ch[1], d.ch[2]);  // level 1
     if (st == ART_OK) st = tap_blocks(8, d.ch[2], d.ch[3]);   // level 2
     if (st == ART_OK && d.arch == ART_NET_TWO_BRANCH) st = sub_blocks(19, d.ach[0], d.ach[1]);
+  }
+  // the FP32 network on the tensor cores: every 3x3 layer's weight parts,
+  // where the widths are ones its kernel takes (else the CUDA-core kernels)
+  if (st == ART_OK && compute_dtype == ART_F32) {
+    auto unet_ok = [&](int levels, const int* ch) {
+      bool ok = ch[0] == 32;  // (the 1x1 head is fused into a 32-channel layer)
+      for (int l = 0; l < levels; ++l) ok = ok && ch[l] % 32 == 0 && (ch[l] <= 64 || ch[l] % 128 == 0);
+      return ok;
+    };
+    bool ok = d.arch == ART_NET_TINY ? d.ch[0] == 32 && d.cout <= 32 : unet_ok(4, d.ch) && d.cout <= 4;
+    if (d.arch == ART_NET_TWO_BRANCH) ok = ok && unet_ok(2, d.ach);
+    for (const ConvLayer& L : ctx->layers) ok = ok && (L.k == 1 || x3_layer_ok(L));
+    auto parts = [&](int li, int cu) -> art_status {  // cu: channels of the upsampled tensor, first in the concatenation
+      ConvLayer& L = ctx->layers[li];
+      art_status s2 = alloc(ctx, &L.wx, x3_weight_elems(L.cout, L.cin - cu, 9), "weight parts");
+      if (s2 != ART_OK) return s2;
+      launch_x3_weights(ctx, L, cu, L.cin - cu, 9, L.wx);
+      if (cu == 0) return ART_OK;
+      if ((s2 = alloc(ctx, &L.wxu, x3_weight_elems(L.cout, cu, 16), "weight parts")) != ART_OK) return s2;
+      launch_x3_weights(ctx, L, 0, cu, 16, L.wxu);
+      return ART_OK;
+    };
+    auto unet_parts = [&](int lb, int levels, const int* ch) -> art_status {
+      art_status s2 = ART_OK;
+      for (int i = 0; i < 4 * levels - 2 && s2 == ART_OK; ++i) {
+        const int dec = i - 2 * levels;  // decoder layers: levels - 2 down to 0, two each
+        s2 = parts(lb + i, dec >= 0 && dec % 2 == 0 ? ch[levels - 1 - dec / 2] : 0);
+      }
+      return s2;
+    };
+    if (ok && d.arch == ART_NET_TINY)
+      for (int i = 0; i < 3 && st == ART_OK; ++i) st = parts(i, 0);
+    else if (ok)
+      st = unet_parts(0, 4, d.ch);
+    if (ok && st == ART_OK && d.arch == ART_NET_TWO_BRANCH) st = unet_parts(15, 2, d.ach);
   }
   if (st != ART_OK) return st;
   ctx->net = d;

@@ -1,7 +1,8 @@
 // Neural shading network (arXiv 2202.05628, Sec. 3.1 "Neural Shading"):
-// layer orchestration and the CUDA-core implicit-GEMM convolution used for the
-// FP32 form.  The BF16 form runs its 3x3 layers on the tensor cores
-// (cnn_tc.cu).
+// layer orchestration and the CUDA-core implicit-GEMM convolutions.  The BF16
+// and FP8 forms run their 3x3 layers on the tensor cores (cnn_tc.cu,
+// cnn_sub.cu), the FP32 form too, as three-part BF16 products (cnn_x3.cu);
+// the CUDA-core kernels take the networks whose widths those do not cover.
 #include <type_traits>
 
 #include "internal.cuh"
@@ -412,13 +413,137 @@ void pack_opacity_input(art_ctx* ctx, int64_t npx, const float* A, const float* 
   ART_LAUNCH(ctx, "pack_opacity_input", kfn, (unsigned)((npx + 255) / 256), 256, 0, npx, A, rgba, x);
 }
 
+// The FP32 network on the tensor cores (cnn_x3.cu): every 3x3 layer from
+// layers[lb] on has its weight parts, which load_shader makes for networks
+// whose widths the kernel takes (x3_net_ok).
+bool has_parts(art_ctx* ctx, int lb) { return lb < (int)ctx->layers.size() && ctx->layers[lb].wx != nullptr; }
+
+// Bytes of unet_x3's parts tensors.
+size_t unet_x3_bytes(int H, int W, int cin, int levels, const int* ch) {
+  size_t t = align256((size_t)H * W * x3_cin_pad(cin) * 6);
+  for (int l = 0; l < levels; ++l) {
+    const size_t px = (size_t)(H >> l) * (W >> l);
+    t += 2 * align256(px * ch[l] * 6);
+    if (l + 1 < levels) t += align256(px / 4 * ch[l] * 6);
+    if (l > 0 && l + 1 < levels) t += align256(px * ch[l] * 6);
+  }
+  return t;
+}
+
+// U-Net of `levels` levels, layers and outputs as in unet_simt: the input is
+// split into parts once, each layer writes its output's parts (the encoders'
+// second layers also their 2x2 maxima), the decoders' first layers read the
+// skip tensor (x-phase split) and the low-resolution tensor in their
+// sub-pixel form, the last layer carries the 1x1 head.  A decoder's first
+// output reuses the space of its level's first encoder output.
+art_status unet_x3(art_ctx* ctx, int H, int W, const float* in, int cin, int lb, int levels, const int* ch, float* out,
+                   int out_ld, int out_off, size_t arena_off) {
+  const size_t need = arena_off + unet_x3_bytes(H, W, cin, levels, ch);
+  if (ensure(ctx, &ctx->d_act, &ctx->d_act_bytes, need, "activations") != ART_OK) return ART_ERR_OOM;
+  size_t off = arena_off;
+  auto take = [&](int l, int c, int shift) {
+    void* p = (char*)ctx->d_act + off;
+    off += align256((size_t)(H >> (l + shift)) * (W >> (l + shift)) * c * 6);
+    return p;
+  };
+  auto L = [&](int i) { return &ctx->layers[lb + i]; };
+  void *a[4] = {}, *b[4] = {};
+  const void* x = take(0, x3_cin_pad(cin), 0);
+  int xc = x3_cin_pad(cin);
+  launch_x3_split(ctx, in, (int64_t)H * W, cin, (__nv_bfloat16*)x);
+  art_status st = ART_OK;
+  int li = 0;
+  for (int l = 0; l < levels; ++l, li += 2) {  // encoder
+    a[l] = take(l, ch[l], 0);
+    b[l] = take(l, ch[l], 0);
+    X3Conv c{};
+    c.layer = L(li);
+    c.in = x;
+    c.cs = xc;
+    c.H = H >> l;
+    c.W = W >> l;
+    c.act = 1;
+    c.planes = a[l];
+    if ((st = launch_x3_conv(ctx, c)) != ART_OK) return st;
+    c.layer = L(li + 1);
+    c.in = a[l];
+    c.cs = ch[l];
+    c.planes = b[l];
+    if (l + 1 < levels) {
+      c.psplit = 1;
+      c.pool = take(l, ch[l], 1);
+    }
+    if ((st = launch_x3_conv(ctx, c)) != ART_OK) return st;
+    x = c.pool;
+    xc = ch[l];
+  }
+  const void* d = b[levels - 1];
+  for (int l = levels - 2; l >= 0; --l, li += 2) {  // decoder: conv over [up2(d), skip], conv
+    X3Conv c{};
+    c.layer = L(li);
+    c.in = b[l];
+    c.cs = ch[l];
+    c.up = d;
+    c.cu = ch[l + 1];
+    c.H = H >> l;
+    c.W = W >> l;
+    c.act = 1;
+    c.planes = a[l];
+    if ((st = launch_x3_conv(ctx, c)) != ART_OK) return st;
+    X3Conv e{};
+    e.layer = L(li + 1);
+    e.in = a[l];
+    e.cs = ch[l];
+    e.H = H >> l;
+    e.W = W >> l;
+    e.act = 1;
+    if (l > 0) {
+      e.planes = take(l, ch[l], 0);
+      d = e.planes;
+    } else {
+      e.out = out;
+      e.head = L(li + 2);
+      e.out_ld = out_ld;
+      e.out_off = out_off;
+    }
+    if ((st = launch_x3_conv(ctx, e)) != ART_OK) return st;
+  }
+  return ART_OK;
+}
+
+// The three-layer network on the tensor cores.
+art_status tiny_x3(art_ctx* ctx, int H, int W, const float* F, float* rgba) {
+  const art_net_desc& nd = ctx->net;
+  const size_t fb = align256((size_t)H * W * x3_cin_pad(nd.cin) * 6), ab = align256((size_t)H * W * nd.ch[0] * 6);
+  if (ensure(ctx, &ctx->d_act, &ctx->d_act_bytes, fb + 2 * ab, "activations") != ART_OK) return ART_ERR_OOM;
+  char* p0 = (char*)ctx->d_act;
+  launch_x3_split(ctx, F, (int64_t)H * W, nd.cin, (__nv_bfloat16*)p0);
+  X3Conv c{};
+  c.H = H;
+  c.W = W;
+  art_status st = ART_OK;
+  for (int i = 0; i < 3 && st == ART_OK; ++i) {
+    c.layer = &ctx->layers[i];
+    c.in = i == 0 ? p0 : p0 + fb + (i - 1) * ab;
+    c.cs = i == 0 ? x3_cin_pad(nd.cin) : nd.ch[0];
+    c.act = i < 2 ? 1 : 2;
+    c.planes = i < 2 ? p0 + fb + i * ab : nullptr;
+    c.out = i < 2 ? nullptr : rgba;
+    c.out_ld = nd.cout;
+    st = launch_x3_conv(ctx, c);
+  }
+  return st;
+}
+
 template <typename TI>
 art_status run_typed(art_ctx* ctx, const ViewParams& v, const void* F, const float* A, float* rgba) {
   const int H = v.H, W = v.W;
   const art_net_desc& nd = ctx->net;
   auto L = [&](int i) -> const ConvLayer& { return ctx->layers[i]; };
   const size_t es = sizeof(TI);
+  const bool x3 = std::is_same<TI, float>::value && has_parts(ctx, 0);
   if (nd.arch == ART_NET_TINY) {
+    if (x3) return tiny_x3(ctx, H, W, (const float*)F, rgba);
     int c = nd.ch[0];
     size_t need = 2 * (size_t)H * W * c * es;
     if (ensure(ctx, &ctx->d_act, &ctx->d_act_bytes, need, "activations") != ART_OK) return ART_ERR_OOM;
@@ -429,15 +554,20 @@ art_status run_typed(art_ctx* ctx, const ViewParams& v, const void* F, const flo
     conv<TI>(ctx, conv_args<TI>(b1, c, 0, nullptr, 0, H, W, L(2), rgba, 2, 1), L(2));
     return ART_OK;
   }
-  if (nd.arch == ART_NET_UNET) return unet_simt<TI>(ctx, H, W, F, nd.cin, 0, 4, nd.ch, rgba, nd.cout, 0, 0);
+  if (nd.arch == ART_NET_UNET) {
+    if (x3) return unet_x3(ctx, H, W, (const float*)F, nd.cin, 0, 4, nd.ch, rgba, nd.cout, 0, 0);
+    return unet_simt<TI>(ctx, H, W, F, nd.cin, 0, 4, nd.ch, rgba, nd.cout, 0, 0);
+  }
   // two branches: appearance F -> I_f (rgba channels 0..2), opacity [A, I_f] -> alpha (channel 3)
-  art_status st = unet_simt<TI>(ctx, H, W, F, nd.cin, 0, 4, nd.ch, rgba, 4, 0, 0);
+  art_status st = x3 ? unet_x3(ctx, H, W, (const float*)F, nd.cin, 0, 4, nd.ch, rgba, 4, 0, 0)
+                     : unet_simt<TI>(ctx, H, W, F, nd.cin, 0, 4, nd.ch, rgba, 4, 0, 0);
   if (st != ART_OK) return st;
   const int64_t npx = (int64_t)H * W;
   const size_t xb = align256((size_t)npx * 4 * es);
-  if (ensure(ctx, &ctx->d_act, &ctx->d_act_bytes, xb + unet_simt_bytes(H, W, 2, nd.ach, es), "activations") != ART_OK)
-    return ART_ERR_OOM;
+  const size_t ub = x3 ? unet_x3_bytes(H, W, 4, 2, nd.ach) : unet_simt_bytes(H, W, 2, nd.ach, es);
+  if (ensure(ctx, &ctx->d_act, &ctx->d_act_bytes, xb + ub, "activations") != ART_OK) return ART_ERR_OOM;
   pack_opacity_input<TI, 4>(ctx, npx, A, rgba, (TI*)ctx->d_act);
+  if (x3) return unet_x3(ctx, H, W, (const float*)ctx->d_act, 4, 15, 2, nd.ach, rgba, 4, 3, xb);
   return unet_simt<TI>(ctx, H, W, ctx->d_act, 4, 15, 2, nd.ach, rgba, 4, 3, xb);
 }
 

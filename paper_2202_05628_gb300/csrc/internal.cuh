@@ -104,6 +104,11 @@ struct ConvLayer {
   // ... of levels 1 and up (the tap-by-tap kernel, TcConv::sub): per output
   // phase [4][cout][9 cs + 4 cu]
   __nv_bfloat16* wtap = nullptr;
+  // FP32 network on the tensor cores (cnn_x3.cu): the weights' BF16 parts
+  // [9][3][cout][cin] (of the skip channels where the layer reads a
+  // concatenation), and [16][3][cout][cin] of the low-resolution channels
+  __nv_bfloat16* wx = nullptr;
+  __nv_bfloat16* wxu = nullptr;
   uint8_t* w8 = nullptr;       // [cout][k*k*cin] E4M3
   float* wscale = nullptr;     // [cout] FP8 per-output-channel scale
 };
@@ -468,6 +473,38 @@ void launch_sub_weights(art_ctx* ctx, const float* w32, int cs, int cu, __nv_bfl
 // taps of the low-resolution part ((oy, ox) in {py - 1, py} x {px - 1, px}).
 void launch_sub_tap_weights(art_ctx* ctx, const float* w32, int cout, int cs, int cu, __nv_bfloat16* wtap);
 art_status launch_sub_conv(art_ctx* ctx, const SubConv& c);
+
+// ---- FP32 convolutions on the tensor cores (cnn_x3.cu)
+// conv3x3 over parts tensors ([y][x][3][c] BF16, c a multiple of 32): H x W
+// output; in = the input [H][W], or with up set (sub-pixel form of
+// conv3x3([up2(up), in])) the skip tensor, x-phase split, and the
+// low-resolution tensor.  Output: planes (parts, [H][W][3][cout], psplit:
+// x-phase split; pool: also its 2x2 maxima), or out (FP32: the 1x1 head's
+// sigmoid outputs, else the layer's own channels; out_ld values per pixel).
+struct X3Conv {
+  const ConvLayer* layer;
+  const void* in;
+  int cs;
+  const void* up = nullptr;
+  int cu = 0;
+  int H, W;
+  int act = 1;
+  void* planes = nullptr;
+  int psplit = 0;
+  void* pool = nullptr;
+  float* out = nullptr;
+  const ConvLayer* head = nullptr;
+  int out_ld = 0, out_off = 0;
+};
+bool x3_layer_ok(const ConvLayer& L);
+int x3_cin_pad(int c);   // stored channels of a parts tensor
+int x3_cout_pad(int c);
+size_t x3_weight_elems(int cout, int cin, int taps);
+// Weight parts of input channels [off, off + cnt): 9 taps, or the decoder's 16 low-resolution ones.
+void launch_x3_weights(art_ctx* ctx, const ConvLayer& L, int off, int cnt, int taps, __nv_bfloat16* out);
+void launch_x3_split(art_ctx* ctx, const float* in, int64_t npx, int c, __nv_bfloat16* out);
+art_status launch_x3_conv(art_ctx* ctx, const X3Conv& c);
+
 void launch_pool_bf16(art_ctx* ctx, const __nv_bfloat16* in, int ld, int ch_off, __nv_bfloat16* out, int H, int W,
                       int C, int psplit = 0);
 void launch_pool_fp8(art_ctx* ctx, const uint8_t* in, int ld, int ch_off, uint8_t* out, int H, int W, int C);
