@@ -986,7 +986,7 @@ art_status art_load_shader(art_ctx* ctx, const art_net_desc* desc, const float* 
   if (st == ART_OK && compute_dtype == ART_F32) {
     auto unet_ok = [&](int levels, const int* ch) {
       bool ok = ch[0] == 32;  // (the 1x1 head is fused into a 32-channel layer)
-      for (int l = 0; l < levels; ++l) ok = ok && ch[l] % 32 == 0 && (ch[l] <= 64 || ch[l] % 128 == 0);
+      for (int l = 0; l < levels; ++l) ok = ok && (ch[l] == 32 || ch[l] % 64 == 0);
       return ok;
     };
     bool ok = d.arch == ART_NET_TINY ? d.ch[0] == 32 && d.cout <= 32 : unet_ok(4, d.ch) && d.cout <= 4;

@@ -7,9 +7,9 @@
 // six BF16 products of which each is exact in FP32.  tcgen05.mma truncates
 // its FP32 sums, so two things keep the error below that of a chain of FP32
 // FMAs: the products x1 w1 go to an accumulator of their own (the others,
-// 2^-8 as large, are summed apart), and no accumulator runs over more than
-// 96 channels x taps: each is read out and added to FP32 registers (rounded
-// to nearest) while the tensor cores fill the other one.  Relative error of
+// 2^-8 as large, are summed apart), and that accumulator never runs over more
+// than 96 channels x taps: it is read out and added to FP32 registers (rounded
+// to nearest) while the tensor cores fill the other row's.  Relative error of
 // a sum over K = 320 / 1152 / 3456 ReLU'd inputs (against FP64): 7e-8 / 9e-8 /
 // 1.4e-7, an FP32 FMA chain 2.2e-7 / 4.1e-7 / 7.3e-7; one accumulator
 // for all six products 2e-6 / 7e-6 / 2e-5.
@@ -24,16 +24,21 @@
 // an input row, which serves the three horizontal taps of both rows; one
 // box the N x 32 x 3 weights of a tap, which serves both rows.  Per tap and
 // 16 channels the parts are stacked along N: x1 meets [w1 w2 w3], x2
-// [w1 w2], x3 [w1] (accumulators a | b | c side by side), so N = 32 costs 144
-// instead of 240 cycles (an MMA takes max(N / 2, 32 + N / 4)); N = 128 folds
-// c into b to fit two sets of accumulators into TMEM.  Warp 0 issues TMA,
-// warp 1 MMAs, warps 2-5 and 6-9 are the two rows' epilogues: they drain
-// their accumulator per (tap row, 32 channels), and at the unit's end add
-// bias, ReLU, split and store through TMA (with the fused 2x2 pooling, or
-// the fused 1x1 head + sigmoid).
+// [w1 w2], x3 [w1] (accumulators a | b | c side by side): N = 32 costs 144
+// instead of 240 cycles, N = 64 208 instead of 288 (an MMA takes
+// max(N / 2, 32 + N / 4)).  Warp 0 issues TMA, warp 1 MMAs, warps 2-5 and 6-9
+// are the two rows' epilogues: they drain their row's a per (tap row, 32
+// channels), and at the unit's end add b and c, the bias, ReLU, split and store
+// through TMA (with the fused 2x2 pooling, or the fused 1x1 head + sigmoid).
+// N = 128 (an eighth fewer MMA cycles) measured slower: its sums fill the
+// registers, its drains outlast the other row's MMAs, and small images have
+// half as many units.
 //
+// Bounds: shared-memory bandwidth (operand reads are ~90 % of it at these N,
+// the TMA boxes come on top) at 50-56 % tensor-pipe time for N = 64; for
+// N = 32 the drain and epilogue latencies between its short blocks (32 %).
 // Measured: FP32 frame of 1M voxels at 1024x1024 10.22 ms with the CUDA-core
-// kernels (36 TFLOP/s) -> 2.37 ms; the U-Net at 424x248 1716 -> 694 us.
+// kernels (36 TFLOP/s) -> 1.96 ms; the U-Net at 424x248 1716 -> 398 us.
 //
 // A result that is not finite (an infinite or NaN input, or parts whose
 // products overflow) is recomputed as the FP32 FMA chain over taps and
@@ -56,21 +61,22 @@ constexpr int kHalo = 130;     // input pixels of a box (128 + 2)
 constexpr int kPlaneA = kHalo * kKCB;
 constexpr int kSlotA = (3 * kPlaneA + 1023) / 1024 * 1024;
 constexpr int kBoxA = 3 * kPlaneA;
+constexpr int kMaxCout = 512;
 constexpr int kOutStage = 3 * 128 * kKCB;  // one group's output tile of 32 channels
 
 template <int N>
 struct Cfg {
   static constexpr int kPlaneB = N * kKCB;
   static constexpr int kSlotB = 3 * kPlaneB;
-  static constexpr int kRegions = N == 128 ? 2 : 3;  // accumulators a | b (| c) per row
-  static constexpr int kSet = kRegions * N;          // TMEM columns of one row
+  static constexpr int kSet = 3 * N;                  // TMEM columns of one row: accumulators a | b | c
+  static constexpr int kScratch = 2 * kSet;           // N = 64: the two rows' finished sums, N columns each
   static constexpr int kTmem = N == 32 ? 256 : 512;
-  static constexpr int kSlotsA = N == 128 ? 3 : 4;
-  static constexpr int kSlotsB = N == 128 ? 4 : (N == 64 ? 5 : 9);
+  static constexpr int kSlotsA = 4;
+  static constexpr int kSlotsB = N == 32 ? 9 : 6;
   static constexpr int kSmem = 1024 + kSlotsA * kSlotA + kSlotsB * kSlotB + 2 * kOutStage +
-                               8 * (2 * (kSlotsA + kSlotsB) + 4) + 16 + 4 * (4 * 32 + 4);
+                               8 * (2 * (kSlotsA + kSlotsB) + 4) + 16 + 16 + 4 * kMaxCout + 4 * (4 * 32 + 4);
 };
-static_assert(Cfg<128>::kSmem <= 232448 && Cfg<64>::kSmem <= 232448 && Cfg<32>::kSmem <= 232448, "shared memory");
+static_assert(Cfg<64>::kSmem <= 232448 && Cfg<32>::kSmem <= 232448, "shared memory");
 
 struct Params {
   int H, W;              // output size
@@ -125,6 +131,38 @@ __device__ __forceinline__ void split3(float x, __nv_bfloat16& a, __nv_bfloat16&
   c = __float2bfloat16_rn(r - __bfloat162float(b));
 }
 
+// The parts of eight non-negative values (o: one 16-byte chunk per part): two
+// values per conversion; values a BF16 rounding would overflow go one by one.
+__device__ __forceinline__ void split3x8(const float* x, uint4 (&o)[3]) {
+  float m = x[0];
+#pragma unroll
+  for (int j = 1; j < 8; ++j) m = fmaxf(m, x[j]);
+  if (m < 3.38e38f) {
+    uint32_t w[3][4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      float a = x[2 * j], b = x[2 * j + 1];
+#pragma unroll
+      for (int pl = 0; pl < 3; ++pl) {
+        const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
+        w[pl][j] = *reinterpret_cast<const uint32_t*>(&h);
+        if (pl < 2) {
+          a -= __uint_as_float(w[pl][j] << 16);
+          b -= __uint_as_float(w[pl][j] & 0xFFFF0000u);
+        }
+      }
+    }
+#pragma unroll
+    for (int pl = 0; pl < 3; ++pl) o[pl] = make_uint4(w[pl][0], w[pl][1], w[pl][2], w[pl][3]);
+  } else {
+    __align__(16) __nv_bfloat16 v[3][8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) split3(x[j], v[0][j], v[1][j], v[2][j]);
+#pragma unroll
+    for (int pl = 0; pl < 3; ++pl) o[pl] = *reinterpret_cast<uint4*>(v[pl]);
+  }
+}
+
 // The output (Y, X, co) as one FP32 FMA chain over taps, then channels (the
 // concatenation [up2(up), in] where there is a low-resolution tensor).
 template <bool SUB>
@@ -147,97 +185,185 @@ __device__ __noinline__ float chain(const Params& p, int co, int Y, int X) {
 }
 
 // One tap of one row: 32 channels of A (three parts, kPlaneA apart) against
-// N x 32 weights (three parts, stacked), into the accumulators at d.
+// N x 32 weights (three parts, stacked), into the accumulators a | b | c at d.
+// kFreshA: the tap starts a K block (a begins anew, b and c go on);
+// kFreshAll: it starts the unit.  Descriptors advance by constants.
+enum Start { kGoOn, kFreshA, kFreshAll };
 template <int N>
-__device__ __forceinline__ void tap_mma(uint32_t d, uint32_t a, uint32_t b, bool first) {
+__device__ __forceinline__ void tap_mma(uint32_t d, uint64_t a1, uint64_t w1, Start start) {
+  constexpr uint64_t kA = kPlaneA >> 4, kB = Cfg<N>::kPlaneB >> 4;
 #pragma unroll
-  for (int kk = 0; kk < kKCB / 32; ++kk) {
-    const uint64_t a1 = umma_desc<kKCB>(a + kk * 32), a2 = umma_desc<kKCB>(a + kPlaneA + kk * 32),
-                   a3 = umma_desc<kKCB>(a + 2 * kPlaneA + kk * 32);
-    const uint64_t w1 = umma_desc<kKCB>(b + kk * 32);
-    const uint32_t acc = (first && kk == 0) ? 0u : 1u;
-    if constexpr (N == 128) {
-      const uint64_t w2 = umma_desc<kKCB>(b + Cfg<N>::kPlaneB + kk * 32),
-                     w3 = umma_desc<kKCB>(b + 2 * Cfg<N>::kPlaneB + kk * 32);
-      umma<false>(d, a1, w1, idesc_bf16(128, 2 * N), acc);  // a += x1 w1, b += x1 w2
-      umma<false>(d + N, a1, w3, idesc_bf16(128, N), 1u);
-      umma<false>(d + N, a2, w1, idesc_bf16(128, N), 1u);
-      umma<false>(d + N, a2, w2, idesc_bf16(128, N), 1u);
-      umma<false>(d + N, a3, w1, idesc_bf16(128, N), 1u);
+  for (int kk = 0; kk < kKCB / 32; ++kk, a1 += 2, w1 += 2) {
+    if (kk == 0 && start == kFreshA) {
+      umma<false>(d, a1, w1, idesc_bf16(128, N), 0u);                // a = x1 w1
+      umma<false>(d + N, a1, w1 + kB, idesc_bf16(128, 2 * N), 1u);   // b, c += x1 (w2, w3)
     } else {
-      umma<false>(d, a1, w1, idesc_bf16(128, 3 * N), acc);          // a, b, c += x1 (w1, w2, w3)
-      umma<false>(d + N, a2, w1, idesc_bf16(128, 2 * N), 1u);       // b, c += x2 (w1, w2)
-      umma<false>(d + 2 * N, a3, w1, idesc_bf16(128, N), 1u);       // c += x3 w1
+      umma<false>(d, a1, w1, idesc_bf16(128, 3 * N), kk == 0 && start == kFreshAll ? 0u : 1u);  // a, b, c += x1 (w1, w2, w3)
+    }
+    umma<false>(d + N, a1 + kA, w1, idesc_bf16(128, 2 * N), 1u);     // b, c += x2 (w1, w2)
+    umma<false>(d + 2 * N, a1 + 2 * kA, w1, idesc_bf16(128, N), 1u);  // c += x3 w1
+  }
+}
+
+// The 32 columns at t and the 32 at u.
+__device__ __forceinline__ void tmem_ld32x2(uint32_t t, uint32_t u, uint32_t (&a)[32], uint32_t (&b)[32]) {
+#define ART_R32(r)                                                                                             \
+  "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),  \
+      "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]),   \
+      "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]),  \
+      "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
+      "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%64];\n"
+      "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%32, %33, %34, %35, %36, %37, %38, %39, %40, %41, %42, %43, %44, %45, "
+      "%46, %47, %48, %49, %50, %51, %52, %53, %54, %55, %56, %57, %58, %59, %60, %61, %62, %63}, [%65];\n"
+      "tcgen05.wait::ld.sync.aligned;"
+      : ART_R32(a), ART_R32(b)
+      : "r"(t), "r"(u)
+      : "memory");
+#undef ART_R32
+}
+
+// 32 values into this warp's lanes of the 32 columns at t.
+__device__ __forceinline__ void tmem_st32(uint32_t t, const float* v) {
+  asm volatile(
+      "tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
+      "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31, %32};" ::"r"(t),
+      "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]), "f"(v[4]), "f"(v[5]), "f"(v[6]), "f"(v[7]), "f"(v[8]), "f"(v[9]),
+      "f"(v[10]), "f"(v[11]), "f"(v[12]), "f"(v[13]), "f"(v[14]), "f"(v[15]), "f"(v[16]), "f"(v[17]), "f"(v[18]),
+      "f"(v[19]), "f"(v[20]), "f"(v[21]), "f"(v[22]), "f"(v[23]), "f"(v[24]), "f"(v[25]), "f"(v[26]), "f"(v[27]),
+      "f"(v[28]), "f"(v[29]), "f"(v[30]), "f"(v[31])
+      : "memory");
+}
+
+// Barrier over the `count` threads (whole warps) that name it.
+__device__ __forceinline__ void bar_sync(int id, int count) {
+  asm volatile("barrier.cta.sync %0, %1;" ::"r"(id), "r"(count) : "memory");
+}
+
+// The sums v of 32 output channels from n0 on of this thread's pixel (Y, X):
+// bias, activation, outputs.
+template <int N, bool SUB>
+__device__ __forceinline__ void finish(const Params& p, float (&v)[32], int n0, int Y, int X, int x0, int yy, int q, int g,
+                                       int gt, bool inside, const float* s_bias, const float* s_head, uint8_t* sO,
+                                       const CUtensorMap* tmO) {
+  uint8_t* st = sO + g * kOutStage;
+  // a sum that is not finite (zero times it is NaN) as the FP32 chain
+  float odd0 = 0.0f, odd1 = 0.0f;
+#pragma unroll
+  for (int j = 0; j < 32; j += 2) {
+    odd0 = fmaf(v[j], 0.0f, odd0);
+    odd1 = fmaf(v[j + 1], 0.0f, odd1);
+  }
+  if (odd0 + odd1 != 0.0f && inside) {
+    float fix[32];
+#pragma unroll
+    for (int j = 0; j < 32; ++j) fix[j] = v[j];
+#pragma unroll 1
+    for (int j = 0; j < 32 && n0 + j < p.cout; ++j)
+      if (fix[j] - fix[j] != 0.0f) fix[j] = chain<SUB>(p, n0 + j, Y, X);
+#pragma unroll
+    for (int j = 0; j < 32; ++j) v[j] = fix[j];
+  }
+#pragma unroll
+  for (int j = 0; j < 32; j += 4) {
+    const float4 b = *reinterpret_cast<const float4*>(s_bias + n0 + j);
+    v[j] += b.x;
+    v[j + 1] += b.y;
+    v[j + 2] += b.z;
+    v[j + 3] += b.w;
+  }
+  if (p.act == 1) {
+#pragma unroll
+    for (int j = 0; j < 32; ++j) v[j] = fmaxf(v[j], 0.0f);
+  }
+  if (p.out) {  // FP32 outputs
+    float* o = p.out + ((size_t)Y * p.W + X) * p.out_ld + p.out_off;
+    if (p.head_w) {
+      float h[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+#pragma unroll
+      for (int j = 0; j < 32; j += 4)
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          const float4 w = *reinterpret_cast<const float4*>(s_head + k * 32 + j);
+          h[k] = fmaf(v[j + 3], w.w, fmaf(v[j + 2], w.z, fmaf(v[j + 1], w.y, fmaf(v[j], w.x, h[k]))));
+        }
+#pragma unroll
+      for (int k = 0; k < 4; ++k) h[k] = 1.0f / (1.0f + expf(-(h[k] + s_head[128 + k])));
+      if (inside) {
+        if (p.out_vec) {
+          *reinterpret_cast<float4*>(o) = make_float4(h[0], h[1], h[2], h[3]);
+        } else {
+#pragma unroll
+          for (int k = 0; k < 4; ++k)
+            if (k < p.out_n) o[k] = h[k];
+        }
+      }
+    } else if (inside) {
+#pragma unroll
+      for (int j = 0; j < 32; ++j)
+        if (n0 + j < p.out_n) o[n0 + j] = p.act == 2 ? 1.0f / (1.0f + expf(-v[j])) : v[j];
     }
   }
-}
-
-// The next accumulator columns of each region (n columns apart) into acc: 16
-// of three regions, or 8 of two (N = 128 has no registers left for more).
-template <int REGIONS>
-struct Drain;
-template <>
-struct Drain<3> {
-  static constexpr int kCols = 16;
-  static __device__ __forceinline__ void add(uint32_t t, uint32_t n, float* acc) {
-    uint32_t a[16], b[16], c[16];
-#define ART_R16(r)                                                                                            \
-  "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]), \
-      "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, "
-        "%15}, [%48];\n"
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, "
-        "%29, %30, %31}, [%49];\n"
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%32, %33, %34, %35, %36, %37, %38, %39, %40, %41, %42, %43, %44, "
-        "%45, %46, %47}, [%50];\n"
-        "tcgen05.wait::ld.sync.aligned;"
-        : ART_R16(a), ART_R16(b), ART_R16(c)
-        : "r"(t), "r"(t + n), "r"(t + 2 * n)
-        : "memory");
-#undef ART_R16
+  if (!p.store) return;
+  // the staging tile is free once its last store has read it
+  if (gt == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+  bar_sync(1 + g, 128);
+  {
+    // chunk k of part pl of this pixel's row: the row's start, and the chunk's swizzled offset in it
+    const int r = p.psplit ? q >> 1 : q, plane = (p.psplit ? 64 : 128) * kKCB;
+    uint8_t* row = st + (p.psplit ? (q & 1) * (kOutStage / 2) : 0) + r * kKCB;
+    const int x = (r >> 1) & 3;
 #pragma unroll
-    for (int j = 0; j < 16; ++j)
-      acc[j] += __uint_as_float(a[j]) + (__uint_as_float(b[j]) + __uint_as_float(c[j]));
-  }
-};
-template <>
-struct Drain<2> {
-  static constexpr int kCols = 8;
-  static __device__ __forceinline__ void add(uint32_t t, uint32_t n, float* acc) {
-    uint32_t a[8], b[8];
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%16];\n"
-        "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%8, %9, %10, %11, %12, %13, %14, %15}, [%17];\n"
-        "tcgen05.wait::ld.sync.aligned;"
-        : "=r"(a[0]), "=r"(a[1]), "=r"(a[2]), "=r"(a[3]), "=r"(a[4]), "=r"(a[5]), "=r"(a[6]), "=r"(a[7]), "=r"(b[0]),
-          "=r"(b[1]), "=r"(b[2]), "=r"(b[3]), "=r"(b[4]), "=r"(b[5]), "=r"(b[6]), "=r"(b[7])
-        : "r"(t), "r"(t + n)
-        : "memory");
+    for (int k = 0; k < 4; ++k) {
+      uint4 o[3];
+      split3x8(v + 8 * k, o);
+      uint8_t* d = row + ((k ^ x) << 4);
 #pragma unroll
-    for (int j = 0; j < 8; ++j) acc[j] += __uint_as_float(a[j]) + __uint_as_float(b[j]);
+      for (int pl = 0; pl < 3; ++pl) *reinterpret_cast<uint4*>(d + pl * plane) = o[pl];
+    }
   }
-};
-
-// Barrier over the first `count` threads that name it (whole warps): true on
-// all of them when ok is true on all of them.
-__device__ __forceinline__ bool bar_and(int id, int count, bool ok) {
-  uint32_t r;
-  asm volatile(
-      "{\n .reg .pred p, q;\n setp.ne.u32 p, %1, 0;\n barrier.cta.red.and.pred q, %2, %3, p;\n selp.u32 %0, 1, 0, q;\n}\n"
-      : "=r"(r)
-      : "r"((uint32_t)ok), "r"(id), "r"(count)
-      : "memory");
-  return r != 0;
-}
-
-// 16-byte chunk k of row q of a 64-byte-swizzled tile (its start 512-byte aligned).
-__device__ __forceinline__ int swz(int q, int k) { return q * 64 + ((k ^ ((q >> 1) & 3)) << 4); }
-
-// Position of pixel q (0 .. 127) of part `plane` in the staged output tile:
-// [part][pixel], or x-phase split [phase][part][pixel / 2].
-__device__ __forceinline__ uint8_t* stage_row(uint8_t* st, int plane, int q, bool psplit, int k) {
-  return psplit ? st + (q & 1) * (kOutStage / 2) + plane * 64 * kKCB + swz(q >> 1, k) : st + plane * 128 * kKCB + swz(q, k);
+  fence_proxy_async_smem();
+  if (p.pool)
+    bar_sync(3, 256);
+  else
+    bar_sync(1 + g, 128);
+  if (gt == 0) {
+    if (p.psplit) {
+      tma_store_5d(tmO, st, n0, x0 >> 1, 0, 0, Y);
+      tma_store_5d(tmO, st + kOutStage / 2, n0, x0 >> 1, 0, 1, Y);
+    } else {
+      tma_store_5d(tmO, st, n0, x0, 0, SUB ? g : 0, Y);
+    }
+    asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+  }
+  if (p.pool) {  // 2x2 maxima of both groups' rows (x-phase split): pooled pixel e / 4, channels 8 (e % 4) .. + 7
+    const int e = g * 128 + gt, pq = e >> 2, k = e & 3;
+    const uint8_t* src = sO + pq * kKCB + ((k ^ ((pq >> 1) & 3)) << 4);
+    float m[8];
+#pragma unroll
+    for (int s = 0; s < 4; ++s) {
+      uint4 w[3];
+#pragma unroll
+      for (int pl = 0; pl < 3; ++pl)
+        w[pl] = *reinterpret_cast<const uint4*>(src + (s >> 1) * kOutStage + (s & 1) * (kOutStage / 2) + pl * 64 * kKCB);
+      const __nv_bfloat16* h = reinterpret_cast<const __nv_bfloat16*>(w);
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        const float f = part_sum(h + j, 8);
+        m[j] = s == 0 ? f : fmaxf(m[j], f);
+      }
+    }
+    const int hx = (x0 >> 1) + pq, hw = p.W >> 1;
+    if (hx < hw && yy < (p.H >> 1)) {
+      uint4 o[3];
+      split3x8(m, o);
+#pragma unroll
+      for (int pl = 0; pl < 3; ++pl)
+        *reinterpret_cast<uint4*>(p.pool + (((size_t)yy * hw + hx) * 3 + pl) * p.cout + n0 + 8 * k) = o[pl];
+    }
+    bar_sync(3, 256);  // (both groups' tiles are read: they may be staged again)
+  }
 }
 
 template <int N, bool SUB>
@@ -260,7 +386,9 @@ __global__ void __launch_bounds__(kThreads, 1)
   uint64_t* acce = accf + 2;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acce + 2);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
-  float* s_head = reinterpret_cast<float*>(tmem_slot + 4);  // [4][32] weights, [4] biases
+  // the layer's biases (read per unit: from global memory their latencies cost ~27 us a unit at N = 128)
+  float* s_bias = reinterpret_cast<float*>((reinterpret_cast<uintptr_t>(tmem_slot + 4) + 15) & ~(uintptr_t)15);
+  float* s_head = s_bias + kMaxCout;  // [4][32] weights, [4] biases
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
@@ -279,6 +407,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     *abort_flag = 0;
     fence_mbar_init();
   }
+  for (int i = threadIdx.x; i < p.n_tiles * N; i += kThreads) s_bias[i] = i < p.cout ? p.bias[i] : 0.0f;
   if (p.head_w)
     for (int i = threadIdx.x; i < 4 * 32 + 4; i += kThreads)  // outputs beyond out_n are zero
       s_head[i] = i < 128 ? (i < p.out_n * 32 ? p.head_w[i] : 0.0f) : (i - 128 < p.out_n ? p.head_b[i - 128] : 0.0f);
@@ -341,14 +470,15 @@ __global__ void __launch_bounds__(kThreads, 1)
       RingPos ra, rb;
       uint32_t aph = 0;  // both rows' accumulators are used once per K block
       bool ok = true;
-      const uint32_t a_base = smem_u32(sA), b_base = smem_u32(sB);
+      const uint64_t a_base = umma_desc<kKCB>(smem_u32(sA)), b_base = umma_desc<kKCB>(smem_u32(sB));
       auto wait_a = [&](const RingPos& r) { ok = ok && mbar_wait(&fullA[r.i], r.ph, abort_flag); };
       auto wait_b = [&](const RingPos& r) { ok = ok && mbar_wait(&fullB[r.i], r.ph, abort_flag); };
       auto wait_acc = [&](int r) { ok = ok && mbar_wait(&acce[r], aph ^ 1u, abort_flag); };
-      auto A = [&](const RingPos& r, int off) { return a_base + (uint32_t)(r.i * kSlotA + off * kKCB); };
-      auto B = [&](const RingPos& r) { return b_base + (uint32_t)(r.i * C::kSlotB); };
+      auto A = [&](const RingPos& r, int off) { return a_base + (uint32_t)((r.i * kSlotA + off * kKCB) >> 4); };
+      auto B = [&](const RingPos& r) { return b_base + (uint32_t)((r.i * C::kSlotB) >> 4); };
       const uint32_t d[2] = {tmem_base, tmem_base + (uint32_t)C::kSet};
       for (int u = blockIdx.x; ok && u < p.n_units && !*abort_flag; u += gridDim.x) {
+        Start start = kFreshAll;  // of a block's first tap
         if constexpr (!SUB) {
           for (int c = 0; ok && c < p.c0; ++c) {
             wait_a(ra);
@@ -360,7 +490,7 @@ __global__ void __launch_bounds__(kThreads, 1)
               for (int dx = 0; dx < 3; ++dx) {  // first row: input row dy of the four
                 wait_b(b);
                 tc_fence_after();
-                if (ok) tap_mma<N>(d[0], A(ra, dx), B(b), dx == 0);
+                if (ok) tap_mma<N>(d[0], A(ra, dx), B(b), dx == 0 ? start : kGoOn);
                 b.next(C::kSlotsB);
               }
               if (!ok) break;
@@ -373,12 +503,13 @@ __global__ void __launch_bounds__(kThreads, 1)
               tc_fence_after();
 #pragma unroll
               for (int dx = 0; dx < 3; ++dx) {  // second row: input row dy + 1
-                tap_mma<N>(d[1], A(ra, dx), B(rb), dx == 0);
+                tap_mma<N>(d[1], A(ra, dx), B(rb), dx == 0 ? start : kGoOn);
                 umma_commit(&emptyB[rb.i]);
                 rb.next(C::kSlotsB);
               }
               umma_commit(&accf[1]);
               aph ^= 1u;
+              start = kFreshA;
             }
             if (!ok) break;
             umma_commit(&emptyA[ra.i]);
@@ -399,7 +530,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             for (int dx = 0; dx < 3; ++dx) {  // even column 2j: input columns 2j - 1, 2j, 2j + 1
               wait_b(b);
               tc_fence_after();
-              if (ok) tap_mma<N>(d[0], dx == 1 ? A(e, 1) : A(o, dx / 2), B(b), dx == 0);
+              if (ok) tap_mma<N>(d[0], dx == 1 ? A(e, 1) : A(o, dx / 2), B(b), dx == 0 ? start : kGoOn);
               b.next(C::kSlotsB);
             }
             if (!ok) break;
@@ -409,7 +540,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             tc_fence_after();
 #pragma unroll
             for (int dx = 0; dx < 3; ++dx) {  // odd column 2j + 1: input columns 2j, 2j + 1, 2j + 2
-              tap_mma<N>(d[1], dx == 1 ? A(o, 1) : A(e, 1 + dx / 2), B(rb), dx == 0);
+              tap_mma<N>(d[1], dx == 1 ? A(o, 1) : A(e, 1 + dx / 2), B(rb), dx == 0 ? start : kGoOn);
               umma_commit(&emptyB[rb.i]);
               rb.next(C::kSlotsB);
             }
@@ -417,6 +548,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             umma_commit(&emptyA[e.i]);
             umma_commit(&emptyA[o.i]);
             aph ^= 1u;
+            start = kFreshA;
           }
           for (int k = 0; ok && k < 2 * p.c1; ++k) {  // low-resolution taps: columns j - 1, j | j, j + 1
             wait_a(ra);
@@ -428,7 +560,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                 wait_b(rb);
                 if (!ok) break;
                 tc_fence_after();
-                tap_mma<N>(d[px], A(ra, px + ox), B(rb), ox == 0);
+                tap_mma<N>(d[px], A(ra, px + ox), B(rb), ox == 0 ? kFreshA : kGoOn);
                 umma_commit(&emptyB[rb.i]);
                 rb.next(C::kSlotsB);
               }
@@ -449,12 +581,12 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int qd = warp & 3;           // TMEM lane quarter this warp may access
     const int q = qd * 32 + lane;      // pixel of the tile
     const int gt = threadIdx.x - 64 - 128 * g;  // thread of the group
-    const uint32_t tq = tmem_base + ((uint32_t)(qd * 32) << 16) + (uint32_t)(g * C::kSet);
-    uint8_t* st = sO + g * kOutStage;
+    const uint32_t tl = tmem_base + ((uint32_t)(qd * 32) << 16);
+    const uint32_t tq = tl + (uint32_t)(g * C::kSet), ts = tl + (uint32_t)(C::kScratch + g * N);
     const int n_blocks = SUB ? 3 * p.c0 + 2 * p.c1 : 3 * p.c0;
     uint32_t aph = 0;
-    bool ok = true;
-    for (int u = blockIdx.x; ok && u < p.n_units; u += gridDim.x) {
+    // (after an abort the loops run on without waiting, so that every thread passes every barrier)
+    for (int u = blockIdx.x; u < p.n_units; u += gridDim.x) {
       const int t = u / p.n_tiles, n0 = (u - t * p.n_tiles) * N;
       const int yy = t / p.tiles_x, x0 = (t - yy * p.tiles_x) * 128;
       const int Y = SUB ? yy : 2 * yy + g, X = SUB ? 2 * (x0 + q) + g : x0 + q;
@@ -462,126 +594,57 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
       for (int j = 0; j < N; ++j) acc[j] = 0.0f;
       for (int k = 0; k < n_blocks; ++k) {
-        // (the group decides together: a thread that gave up must not leave the others at a barrier)
-        if (!(ok = bar_and(1 + g, 128, mbar_wait(&accf[g], aph, abort_flag)))) break;
+        if (!*abort_flag) mbar_wait(&accf[g], aph, abort_flag);
         tc_fence_after();
+        if constexpr (N == 32) {
+          uint32_t a[32];
+          tmem_ld32(tq, a);
 #pragma unroll
-        for (int c = 0; c < N; c += Drain<C::kRegions>::kCols) Drain<C::kRegions>::add(tq + (uint32_t)c, N, acc + c);
+          for (int j = 0; j < 32; ++j) acc[j] += __uint_as_float(a[j]);
+        } else {
+          uint32_t a[32], b[32];
+          tmem_ld32x2(tq, tq + 32, a, b);
+#pragma unroll
+          for (int j = 0; j < 32; ++j) {
+            acc[j] += __uint_as_float(a[j]);
+            acc[32 + j] += __uint_as_float(b[j]);
+          }
+        }
+        if (k == n_blocks - 1) {  // the corrections, summed over the whole unit
+#pragma unroll
+          for (int c = 0; c < N; c += 32) {
+            uint32_t a[32], b[32];
+            tmem_ld32x2(tq + (uint32_t)(N + c), tq + (uint32_t)(2 * N + c), a, b);
+#pragma unroll
+            for (int j = 0; j < 32; ++j) acc[c + j] += __uint_as_float(a[j]) + __uint_as_float(b[j]);
+          }
+        }
         tc_fence_before();
         mbar_arrive(&acce[g]);
         aph ^= 1u;
       }
-      if (p.pool) ok = bar_and(3, 256, ok);
-      if (!ok) break;
+      // The sums of N = 64 pass through TMEM, so that one copy of the code below
+      // takes both groups of 32 channels: unrolled over registers it runs once
+      // per unit out of a cold instruction cache.
+      if constexpr (N > 32) {
+#pragma unroll
+        for (int c = 0; c < N; c += 32) tmem_st32(ts + (uint32_t)c, acc + c);
+        tmem_wait_st();
+      }
       const bool inside = Y < p.H && X < p.W;
-      if (!inside) {
-#pragma unroll
-        for (int j = 0; j < N; ++j) acc[j] = 0.0f;
-      }
-      // bias; a sum that is not finite (its difference with itself is not zero) as the FP32 chain
-      float odd = 0.0f;
-#pragma unroll
-      for (int j = 0; j < N; ++j) odd += acc[j] - acc[j];
-      if (odd != 0.0f) {
-        float fix[N];
-#pragma unroll
-        for (int j = 0; j < N; ++j) fix[j] = acc[j];
 #pragma unroll 1
-        for (int j = 0; j < N && n0 + j < p.cout; ++j)
-          if (fix[j] - fix[j] != 0.0f) fix[j] = chain<SUB>(p, n0 + j, Y, X);
+      for (int c = 0; c < N; c += 32) {
+        float v[32];
+        if constexpr (N > 32) {
+          uint32_t a[32];
+          tmem_ld32(ts + (uint32_t)c, a);
 #pragma unroll
-        for (int j = 0; j < N; ++j) acc[j] = fix[j];
-      }
+          for (int j = 0; j < 32; ++j) v[j] = __uint_as_float(a[j]);
+        } else {
 #pragma unroll
-      for (int j = 0; j < N; ++j) {
-        const float b = n0 + j < p.cout ? __ldg(p.bias + n0 + j) : 0.0f;
-        acc[j] += b;
-        if (p.act == 1) acc[j] = fmaxf(acc[j], 0.0f);
-      }
-      if (p.out) {  // FP32 outputs
-        float* o = p.out + ((size_t)Y * p.W + X) * p.out_ld + p.out_off;
-        if (p.head_w) {
-          float v[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-#pragma unroll
-          for (int j = 0; j < 32; ++j)
-#pragma unroll
-            for (int k = 0; k < 4; ++k) v[k] = fmaf(acc[j], s_head[k * 32 + j], v[k]);
-#pragma unroll
-          for (int k = 0; k < 4; ++k) v[k] = 1.0f / (1.0f + expf(-(v[k] + s_head[128 + k])));
-          if (inside) {
-            if (p.out_vec) {
-              *reinterpret_cast<float4*>(o) = make_float4(v[0], v[1], v[2], v[3]);
-            } else {
-#pragma unroll
-              for (int k = 0; k < 4; ++k)
-                if (k < p.out_n) o[k] = v[k];
-            }
-          }
-        } else if (inside) {
-#pragma unroll
-          for (int j = 0; j < N; ++j)
-            if (n0 + j < p.out_n) o[n0 + j] = p.act == 2 ? 1.0f / (1.0f + expf(-acc[j])) : acc[j];
+          for (int j = 0; j < 32; ++j) v[j] = acc[j];
         }
-      }
-      if (p.store) {
-#pragma unroll
-        for (int c = 0; c < N; c += 32) {
-          // the staging tile is free once its last store has read it
-          if (gt == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
-          bar_and(1 + g, 128, true);
-#pragma unroll
-          for (int k = 0; k < 4; ++k) {
-            __align__(16) __nv_bfloat16 v[3][8];
-#pragma unroll
-            for (int j = 0; j < 8; ++j) split3(acc[c + 8 * k + j], v[0][j], v[1][j], v[2][j]);
-#pragma unroll
-            for (int pl = 0; pl < 3; ++pl)
-              *reinterpret_cast<uint4*>(stage_row(st, pl, q, p.psplit != 0, k)) = *reinterpret_cast<uint4*>(v[pl]);
-          }
-          fence_proxy_async_smem();
-          if (p.pool)
-            bar_and(3, 256, true);
-          else
-            bar_and(1 + g, 128, true);
-          if (gt == 0) {
-            if (p.psplit) {
-              tma_store_5d(&tmO, st, n0 + c, x0 >> 1, 0, 0, Y);
-              tma_store_5d(&tmO, st + kOutStage / 2, n0 + c, x0 >> 1, 0, 1, Y);
-            } else {
-              tma_store_5d(&tmO, st, n0 + c, x0, 0, SUB ? g : 0, Y);
-            }
-            asm volatile("cp.async.bulk.commit_group;" ::: "memory");
-          }
-          if (p.pool) {  // 2x2 maxima of both groups' rows: pooled pixel e / 4, channels 8 (e % 4) .. + 7
-            const int e = g * 128 + gt, pq = e >> 2, k = e & 3;
-            float m[8];
-#pragma unroll
-            for (int s = 0; s < 4; ++s) {
-              uint4 w[3];
-#pragma unroll
-              for (int pl = 0; pl < 3; ++pl)
-                w[pl] = *reinterpret_cast<const uint4*>(
-                    stage_row(sO + (s >> 1) * kOutStage, pl, 2 * pq + (s & 1), p.psplit != 0, k));
-              const __nv_bfloat16* h = reinterpret_cast<const __nv_bfloat16*>(w);
-#pragma unroll
-              for (int j = 0; j < 8; ++j) {
-                const float f = part_sum(h + j, 8);
-                m[j] = s == 0 ? f : fmaxf(m[j], f);
-              }
-            }
-            const int hx = (x0 >> 1) + pq, hw = p.W >> 1;
-            if (hx < hw && yy < (p.H >> 1)) {
-              __align__(16) __nv_bfloat16 v[3][8];
-#pragma unroll
-              for (int j = 0; j < 8; ++j) split3(m[j], v[0][j], v[1][j], v[2][j]);
-#pragma unroll
-              for (int pl = 0; pl < 3; ++pl)
-                *reinterpret_cast<uint4*>(p.pool + (((size_t)yy * hw + hx) * 3 + pl) * p.cout + n0 + c + 8 * k) =
-                    *reinterpret_cast<uint4*>(v[pl]);
-            }
-            bar_and(3, 256, true);  // (both groups' tiles are read: they may be staged again)
-          }
-        }
+        finish<N, SUB>(p, v, n0 + c, Y, X, x0, yy, q, g, gt, inside, s_bias, s_head, sO, &tmO);
       }
     }
     if (gt == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
@@ -654,8 +717,6 @@ __global__ void __launch_bounds__(256) x3_split_kernel(const float* __restrict__
       *reinterpret_cast<uint4*>(out + (px * 3 + pl) * cp + c0) = *reinterpret_cast<uint4*>(v[pl]);
   }
 }
-
-int n_of(int cout) { return cout <= 32 ? 32 : (cout == 64 ? 64 : 128); }
 
 // Parts tensor as (channel, x, part, x phase, y): ph = 1, 2 phases stored
 // one after the other per row (split), or 2 interleaved ones (pixel 2x + phase).
@@ -744,7 +805,7 @@ int x3_cin_pad(int c) { return (c + kKC - 1) / kKC * kKC; }
 int x3_cout_pad(int c) { return c <= 32 ? 32 : c; }
 
 bool x3_layer_ok(const ConvLayer& L) {
-  return L.k == 3 && (L.cout <= 32 || L.cout == 64 || L.cout % 128 == 0) && tensor_map_encoder() != nullptr;
+  return L.k == 3 && L.cout <= kMaxCout && (L.cout <= 32 || L.cout % 64 == 0) && tensor_map_encoder() != nullptr;
 }
 
 size_t x3_weight_elems(int cout, int cin, int taps) { return (size_t)taps * 3 * x3_cout_pad(cout) * x3_cin_pad(cin); }
@@ -765,11 +826,8 @@ void launch_x3_split(art_ctx* ctx, const float* in, int64_t npx, int c, __nv_bfl
 }
 
 art_status launch_x3_conv(art_ctx* ctx, const X3Conv& c) {
-  switch (n_of(c.layer->cout)) {
-    case 32: return c.up ? launch_n<32, true>(ctx, c) : launch_n<32, false>(ctx, c);
-    case 64: return c.up ? launch_n<64, true>(ctx, c) : launch_n<64, false>(ctx, c);
-    default: return c.up ? launch_n<128, true>(ctx, c) : launch_n<128, false>(ctx, c);
-  }
+  if (c.layer->cout <= 32) return c.up ? launch_n<32, true>(ctx, c) : launch_n<32, false>(ctx, c);
+  return c.up ? launch_n<64, true>(ctx, c) : launch_n<64, false>(ctx, c);
 }
 
 }  // namespace art

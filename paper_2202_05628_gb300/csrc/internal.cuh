@@ -479,7 +479,7 @@ art_status launch_sub_conv(art_ctx* ctx, const SubConv& c);
 // output; in = the input [H][W], or with up set (sub-pixel form of
 // conv3x3([up2(up), in])) the skip tensor, x-phase split, and the
 // low-resolution tensor.  Output: planes (parts, [H][W][3][cout], psplit:
-// x-phase split; pool: also its 2x2 maxima), or out (FP32: the 1x1 head's
+// x-phase split; pool: also the 2x2 maxima of a split output), or out (FP32: the 1x1 head's
 // sigmoid outputs, else the layer's own channels; out_ld values per pixel).
 struct X3Conv {
   const ConvLayer* layer;
