@@ -181,7 +181,7 @@ void free_all(art_ctx* ctx) {
                   ctx->d_rec, ctx->d_geo, ctx->d_rect, ctx->d_q, ctx->d_cnt, ctx->d_keys,
                   ctx->d_vals, ctx->d_sort_tmp, ctx->d_ranges,
                   ctx->d_status, ctx->d_F, ctx->d_A, ctx->d_rgba, ctx->d_act, ctx->d_sk, ctx->d_sv,
-                  ctx->d_shist, ctx->d_sbsum, ctx->d_gN, ctx->d_f8_scale, ctx->d_f8_amax, ctx->d_prop_img,
+                  ctx->d_slook, ctx->d_scounts, ctx->d_gN, ctx->d_f8_scale, ctx->d_f8_amax, ctx->d_prop_img,
                   ctx->d_prop_f32, ctx->d_pose_bias, ctx->d_bins, ctx->d_thist, ctx->d_hbin, ctx->d_htau, ctx->d_fbq,
                   ctx->d_seg, ctx->d_items, ctx->d_multi, ctx->d_part, ctx->d_fbq2, ctx->d_tcount, ctx->d_toff,
                   ctx->d_sortlist, ctx->d_scan_state, ctx->d_agroups, ctx->d_sh, ctx->d_sh_rot, ctx->d_rect_v,
@@ -1188,7 +1188,7 @@ art_status art_sync_status(art_ctx* ctx, art_stats* out) {
     return r;
   }
   if (h[kStScanError]) {
-    art_status r = fail(ctx, ART_ERR_CUDA, "binning: %llu tile-scan blocks timed out waiting for a predecessor",
+    art_status r = fail(ctx, ART_ERR_CUDA, "binning or sort: %llu look-backs timed out waiting for a predecessor",
                         h[kStScanError]);
     cudaMemsetAsync(ctx->d_status + kStScanError, 0, sizeof(unsigned long long), ctx->stream);
     cudaStreamSynchronize(ctx->stream);
@@ -1233,14 +1233,11 @@ art_status art_sort_pairs(art_ctx* ctx, uint32_t* keys, uint32_t* vals, int64_t 
   if (n > ctx->sort_cap) {
     if ((st = alloc(ctx, &ctx->d_sk, (size_t)n, "sort scratch keys")) != ART_OK) return st;
     if ((st = alloc(ctx, &ctx->d_sv, (size_t)n, "sort scratch values")) != ART_OK) return st;
-    size_t hw = sort_hist_words(n);
-    if ((st = alloc(ctx, &ctx->d_shist, hw, "sort histogram")) != ART_OK) return st;
-    if ((st = alloc(ctx, &ctx->d_sbsum, scan_block_words((int64_t)hw), "sort block sums")) != ART_OK) return st;
+    if ((st = alloc(ctx, &ctx->d_slook, sort_look_words(n), "sort look-back words")) != ART_OK) return st;
+    if ((st = alloc(ctx, &ctx->d_scounts, sort_count_words(), "sort counts")) != ART_OK) return st;
     ctx->sort_cap = n;
   }
-  unsigned long long* cnt = ctx->d_status + 6;
-  launch_set_word(ctx, cnt, (unsigned long long)n);
-  int where = launch_sort_bufs(ctx, keys, vals, ctx->d_sk, ctx->d_sv, n, cnt, key_bits, ctx->d_shist, ctx->d_sbsum);
+  const int where = launch_sort(ctx, keys, vals, ctx->d_sk, ctx->d_sv, n, key_bits, ctx->d_scounts, ctx->d_slook);
   if (where == 1) {
     cudaMemcpyAsync(keys, ctx->d_sk, sizeof(uint32_t) * (size_t)n, cudaMemcpyDeviceToDevice, ctx->stream);
     cudaMemcpyAsync(vals, ctx->d_sv, sizeof(uint32_t) * (size_t)n, cudaMemcpyDeviceToDevice, ctx->stream);

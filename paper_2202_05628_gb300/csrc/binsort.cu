@@ -5,21 +5,13 @@
 #include <cuda.h>
 #include <cudaTypedefs.h>
 
+#include <algorithm>
 #include <mutex>
 
 #include "internal.cuh"
 
 namespace art {
 namespace {
-
-constexpr int kScanThreads = 256;
-constexpr int kScanItems = 8;                       // per thread
-constexpr int kScanBlock = kScanThreads * kScanItems;  // 2048
-constexpr int kSortThreads = 256;
-constexpr int kSortRounds = 16;
-constexpr int kSortBlock = kSortThreads * kSortRounds;  // 4096 keys per block
-constexpr int kRadixBits = 8;
-constexpr int kRadix = 1 << kRadixBits;
 
 // Block-wide exclusive scan of one value per thread (256 threads).
 __device__ uint32_t block_exclusive_scan(uint32_t v, uint32_t* total) {
@@ -50,167 +42,225 @@ __device__ uint32_t block_exclusive_scan(uint32_t v, uint32_t* total) {
   return base + x - v;
 }
 
-// Sum of each block of kScanBlock elements.
-__global__ void __launch_bounds__(kScanThreads) block_sum_kernel(const uint32_t* __restrict__ in, int64_t n,
-                                                                 const unsigned long long* __restrict__ n_dev,
-                                                                 uint32_t* __restrict__ bsum) {
-  if (n_dev) n = (int64_t)min((unsigned long long)n, *n_dev);
-  int64_t base = (int64_t)blockIdx.x * kScanBlock;
-  uint32_t s = 0;
-#pragma unroll
-  for (int k = 0; k < kScanItems; ++k) {
-    int64_t i = base + (int64_t)k * kScanThreads + threadIdx.x;
-    if (i < n) s += in[i];
-  }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-  __shared__ uint32_t ws[kScanThreads / 32];
-  if ((threadIdx.x & 31) == 0) ws[threadIdx.x >> 5] = s;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    uint32_t t = 0;
-    for (int w = 0; w < kScanThreads / 32; ++w) t += ws[w];
-    bsum[blockIdx.x] = t;
-  }
-}
-
-// Exclusive scan of nb block sums in one block of 1024 threads (nb <= 1024 *
-// 16); writes the grand total to *total (64-bit) when non-null.
-__global__ void __launch_bounds__(1024) scan_bsum_kernel(uint32_t* __restrict__ bsum, int nb,
-                                                         unsigned long long* __restrict__ total) {
-  constexpr int kPer = 16;
-  __shared__ uint32_t warp_sums[32];
-  uint32_t v[kPer];
-  uint32_t s = 0;
-  int base = threadIdx.x * kPer;
-#pragma unroll
-  for (int k = 0; k < kPer; ++k) {
-    v[k] = (base + k < nb) ? bsum[base + k] : 0u;
-    s += v[k];
-  }
-  int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  uint32_t x = s;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
-    if (lane >= o) x += y;
-  }
-  if (lane == 31) warp_sums[wid] = x;
-  __syncthreads();
-  if (wid == 0) {
-    uint32_t w = warp_sums[lane];
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      uint32_t y = __shfl_up_sync(0xffffffffu, w, o);
-      if (lane >= o) w += y;
-    }
-    warp_sums[lane] = w;
-  }
-  __syncthreads();
-  uint32_t run = (wid > 0 ? warp_sums[wid - 1] : 0u) + x - s;
-#pragma unroll
-  for (int k = 0; k < kPer; ++k) {
-    if (base + k < nb) bsum[base + k] = run;
-    run += v[k];
-  }
-  if (total && threadIdx.x == 1023) *total = (unsigned long long)run;
-}
-
-// Exclusive scan of `in` into `out` given scanned block sums.
-// (in and out may alias: each thread reads its own items before writing them)
-__global__ void __launch_bounds__(kScanThreads) scan_apply_kernel(const uint32_t* in, uint32_t* out, int64_t n,
-                                                                  const uint32_t* __restrict__ bsum) {
-  int64_t base = (int64_t)blockIdx.x * kScanBlock + (int64_t)threadIdx.x * kScanItems;
-  uint32_t v[kScanItems];
-  uint32_t s = 0;
-#pragma unroll
-  for (int k = 0; k < kScanItems; ++k) {
-    v[k] = (base + k < n) ? in[base + k] : 0u;
-    s += v[k];
-  }
-  uint32_t run = block_exclusive_scan(s, nullptr) + bsum[blockIdx.x];
-#pragma unroll
-  for (int k = 0; k < kScanItems; ++k) {
-    if (base + k < n) out[base + k] = run;
-    run += v[k];
-  }
-}
-
 // ---------------------------------------------------------------- radix sort
+//
+// Stable LSD radix sort of 32-bit pairs, eight bits a pass: one kernel counts
+// every pass's digits over all keys, then one kernel per pass ranks, exchanges
+// and scatters.  A block takes the next tile of 4096 pairs (a ticket, so every
+// predecessor is running), ranks its pairs by warp matches, publishes its digit
+// counts, and thread d looks back over the earlier tiles' counts of digit d,
+// sixteen of them per round: all of a small sort's tiles run at once, so the
+// nearest published prefix is far at first and a walk one tile at a time would
+// take as many memory latencies as there are tiles.  The pairs are brought into
+// digit order in shared memory meanwhile, so that runs of a digit are stored
+// contiguously.
+constexpr int kSortThreads = 256;
+constexpr int kSortWarps = kSortThreads / 32;
+constexpr int kSortRounds = 16;
+constexpr int kSortTile = kSortThreads * kSortRounds;  // 4096 pairs per tile
+constexpr int kRadixBits = 8;
+constexpr int kRadix = 1 << kRadixBits;
+constexpr int kMaxPasses = 4;
+constexpr int kLookBack = 16;            // predecessors read per look-back round
+constexpr int kCountReplicas = 4;        // digit counters per block of the count (lanes of a warp often share a digit)
+constexpr long long kSortSpin = 1 << 22;  // look-back polls before a block gives up
 
-// number of keys: the device count word, clamped to the capacity
-__device__ __forceinline__ int64_t num_keys(const unsigned long long* st, int64_t cap) {
-  unsigned long long m = *st;
-  return (int64_t)(m < (unsigned long long)cap ? m : (unsigned long long)cap);
-}
+// What a tile has published of a digit in a pass: nothing, its own count, or
+// the count of all tiles up to it.  The tag names the pass, so one array
+// (zeroed once per sort) serves all passes.  32-bit words hold counts of sorts
+// below 2^28 pairs.
+template <typename S>
+struct LookWord;
+template <>
+struct LookWord<uint32_t> {
+  static constexpr int kShift = 28;
+};
+template <>
+struct LookWord<unsigned long long> {
+  static constexpr int kShift = 32;
+};
+constexpr int64_t kSmallSort = (int64_t)1 << 28;
 
-// Digit histogram of each 4096-key block; layout hist[digit * nb + block].
-__global__ void __launch_bounds__(kSortThreads) radix_hist_kernel(const uint32_t* __restrict__ keys, int64_t cap,
-                                                                  const unsigned long long* __restrict__ st,
-                                                                  int shift, int nb, uint32_t* __restrict__ hist) {
-  __shared__ uint32_t h[kRadix];
-  h[threadIdx.x] = 0;
+// Counters of a sort: [kMaxPasses][kRadix] digit counts, then a tile ticket per pass (zeroed before).
+constexpr int kCountWords = kMaxPasses * kRadix + kMaxPasses;
+
+// Digit counts of all passes, and the look-back words zeroed.
+__global__ void __launch_bounds__(kSortThreads) radix_count_kernel(const uint32_t* __restrict__ keys, int64_t n,
+                                                                   int passes, uint32_t* __restrict__ counts,
+                                                                   uint32_t* __restrict__ look, int64_t look_words) {
+  __shared__ uint32_t h[kCountReplicas][kMaxPasses * kRadix];
+  for (int k = threadIdx.x; k < kCountReplicas * kMaxPasses * kRadix; k += kSortThreads) (&h[0][0])[k] = 0;
+  const int64_t tid = (int64_t)blockIdx.x * kSortThreads + threadIdx.x, nth = (int64_t)gridDim.x * kSortThreads;
+  for (int64_t k = tid; k < look_words; k += nth) look[k] = 0;
   __syncthreads();
-  int64_t n = num_keys(st, cap);
-  int64_t base = (int64_t)blockIdx.x * kSortBlock;
-  if (base < n) {
-#pragma unroll 4
-    for (int r = 0; r < kSortRounds; ++r) {
-      int64_t i = base + (int64_t)r * kSortThreads + threadIdx.x;
-      if (i < n) atomicAdd(&h[(keys[i] >> shift) & (kRadix - 1)], 1u);
-    }
+  uint32_t* mine = h[threadIdx.x % kCountReplicas];
+  for (int64_t i0 = tid; i0 < n; i0 += 8 * nth) {  // eight loads in flight
+    uint32_t k[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) k[j] = i0 + j * nth < n ? keys[i0 + j * nth] : 0u;
+#pragma unroll
+    for (int j = 0; j < 8; ++j)
+      if (i0 + j * nth < n)
+        for (int q = 0; q < passes; ++q) atomicAdd(&mine[q * kRadix + ((k[j] >> (q * kRadixBits)) & (kRadix - 1))], 1u);
   }
   __syncthreads();
-  hist[(int64_t)threadIdx.x * nb + blockIdx.x] = h[threadIdx.x];
+  for (int k = threadIdx.x; k < passes * kRadix; k += kSortThreads) {
+    uint32_t c = 0;
+#pragma unroll
+    for (int r = 0; r < kCountReplicas; ++r) c += h[r][k];
+    if (c) atomicAdd(counts + k, c);
+  }
 }
 
-// Stable scatter of each block's keys by digit, using the scanned histogram.
-__global__ void __launch_bounds__(kSortThreads) radix_scatter_kernel(
-    const uint32_t* __restrict__ kin, const uint32_t* __restrict__ vin, uint32_t* __restrict__ kout,
-    uint32_t* __restrict__ vout, int64_t cap, const unsigned long long* __restrict__ st, int shift, int nb,
-    const uint32_t* __restrict__ hist) {
-  constexpr int kWarps = kSortThreads / 32;
-  __shared__ uint32_t run[kRadix];        // running position of each digit
-  __shared__ uint32_t wh[kWarps][kRadix];  // per-warp digit counts -> offsets
-  __shared__ uint32_t rt[kRadix];         // round totals
-  int64_t n = num_keys(st, cap);
-  int64_t base = (int64_t)blockIdx.x * kSortBlock;
-  if (base >= n) return;
-  int t = threadIdx.x, lane = t & 31, w = t >> 5;
-  run[t] = hist[(int64_t)t * nb + blockIdx.x];
-  unsigned lt = (1u << lane) - 1u;
+template <typename S>
+__global__ void __launch_bounds__(kSortThreads) radix_pass_kernel(const uint32_t* __restrict__ kin,
+                                                                  const uint32_t* __restrict__ vin,
+                                                                  uint32_t* __restrict__ kout,
+                                                                  uint32_t* __restrict__ vout, int64_t n, int pass,
+                                                                  uint32_t* __restrict__ counts, S* look,
+                                                                  unsigned long long* __restrict__ err) {
+  ART_PDL_ENTRY();
+  constexpr int kShift = LookWord<S>::kShift;
+  __shared__ uint32_t wh[kSortWarps][kRadix];  // per warp: digit counts, then offsets within the tile's digit
+  __shared__ uint32_t s_start[kRadix];         // the tile's digit starts
+  __shared__ uint32_t s_base[kRadix];          // output position of the digit's pair p of the tile: s_base + p
+  __shared__ uint32_t s_key[kSortTile], s_val[kSortTile];
+  __shared__ uint32_t s_tile;
+  const int t = threadIdx.x, lane = t & 31, w = t >> 5;
+  if (t == 0) s_tile = atomicAdd(counts + kMaxPasses * kRadix + pass, 1u);
+#pragma unroll
+  for (int k = 0; k < kSortWarps; ++k) wh[k][t] = 0;
+  __syncthreads();
+  const uint32_t tile = s_tile;
+  const int64_t base = (int64_t)tile * kSortTile;
+  const int m = (int)min((int64_t)kSortTile, n - base);
+  const int shift = pass * kRadixBits;
+  // warp w's pairs: [512 w, 512 w + 512) of the tile, 32 consecutive ones a round
+  uint32_t key[kSortRounds], val[kSortRounds], rank[kSortRounds];
+#pragma unroll
   for (int r = 0; r < kSortRounds; ++r) {
-#pragma unroll
-    for (int k = 0; k < kWarps; ++k) wh[k][t] = 0;
-    __syncthreads();
-    int64_t i = base + (int64_t)r * kSortThreads + t;
-    bool valid = i < n;
-    uint32_t key = valid ? kin[i] : 0u;
-    uint32_t val = valid ? vin[i] : 0u;
-    uint32_t d = valid ? ((key >> shift) & (kRadix - 1)) : (uint32_t)kRadix;
-    unsigned peers = __match_any_sync(0xffffffffu, d);
-    uint32_t rank = __popc(peers & lt);
-    if (valid && rank == 0) wh[w][d] = __popc(peers);
-    __syncthreads();
-    {
-      uint32_t s = 0;
-#pragma unroll
-      for (int k = 0; k < kWarps; ++k) {
-        uint32_t c = wh[k][t];
-        wh[k][t] = s;
-        s += c;
-      }
-      rt[t] = s;
-    }
-    __syncthreads();
-    if (valid) {
-      uint32_t pos = run[d] + wh[w][d] + rank;
-      kout[pos] = key;
-      vout[pos] = val;
-    }
-    __syncthreads();
-    run[t] += rt[t];
+    const int i = w * (32 * kSortRounds) + r * 32 + lane;
+    key[r] = i < m ? kin[base + i] : 0u;
+    val[r] = i < m ? vin[base + i] : 0u;
   }
+  const unsigned lt = (1u << lane) - 1u;
+#pragma unroll
+  for (int r = 0; r < kSortRounds; ++r) {
+    const bool in = w * (32 * kSortRounds) + r * 32 + lane < m;
+    const uint32_t d = in ? (key[r] >> shift) & (kRadix - 1) : (uint32_t)kRadix;
+    const unsigned peers = __match_any_sync(0xffffffffu, d);
+    const int leader = __ffs(peers) - 1;
+    uint32_t before = 0;
+    if (in && lane == leader) {
+      before = wh[w][d];
+      wh[w][d] = before + __popc(peers);
+    }
+    __syncwarp();
+    rank[r] = __shfl_sync(0xffffffffu, before, leader) + __popc(peers & lt);
+  }
+  __syncthreads();
+  // thread t = digit t: offsets of the warps, the tile's count, published
+  uint32_t c = 0;
+#pragma unroll
+  for (int k = 0; k < kSortWarps; ++k) {
+    const uint32_t x = wh[k][t];
+    wh[k][t] = c;
+    c += x;
+  }
+  const S tag_own = (S)(pass * 4 + 1), tag_all = (S)(pass * 4 + 2);
+  volatile S* mine = look + (size_t)tile * kRadix + t;
+  *mine = ((tile == 0 ? tag_all : tag_own) << kShift) | (S)c;
+  const uint32_t start = block_exclusive_scan(c, nullptr);
+  s_start[t] = start;
+  const uint32_t first = block_exclusive_scan(counts[pass * kRadix + t], nullptr);  // (its barriers publish s_start)
+  // the tile in digit order, in shared memory
+#pragma unroll
+  for (int r = 0; r < kSortRounds; ++r) {
+    if (w * (32 * kSortRounds) + r * 32 + lane < m) {
+      const uint32_t d = (key[r] >> shift) & (kRadix - 1);
+      const uint32_t pos = s_start[d] + wh[w][d] + rank[r];
+      s_key[pos] = key[r];
+      s_val[pos] = val[r];
+    }
+  }
+  // look back over the earlier tiles' counts of this digit
+  uint32_t prev = 0;
+  int64_t q = (int64_t)tile - 1;
+  long long spin = 0;
+  while (q >= 0) {
+    S x[kLookBack];
+#pragma unroll
+    for (int j = 0; j < kLookBack; ++j)
+      x[j] = q - j >= 0 ? *reinterpret_cast<const volatile S*>(look + (size_t)(q - j) * kRadix + t) : (S)0;
+    int used = 0;
+    bool end = false;
+#pragma unroll
+    for (int j = 0; j < kLookBack; ++j) {
+      if (used == j && !end) {  // (all nearer ones were there)
+        const S tag = x[j] >> kShift;
+        if (tag == tag_own || tag == tag_all) {
+          prev += (uint32_t)(x[j] & ((((S)1) << kShift) - 1));
+          ++used;
+          end = tag == tag_all;
+        }
+      }
+    }
+    if (end) break;
+    q -= used;
+    if (used == 0 && ++spin > kSortSpin) {
+      if (err) atomicAdd(err, 1ull);
+      break;
+    }
+  }
+  if (tile > 0) *mine = (tag_all << kShift) | (S)(prev + c);
+  s_base[t] = first + prev - start;
+  __syncthreads();
+  for (int p = t; p < m; p += kSortThreads) {
+    const uint32_t k = s_key[p];
+    const uint32_t o = s_base[(k >> shift) & (kRadix - 1)] + (uint32_t)p;
+    kout[o] = k;
+    vout[o] = s_val[p];
+  }
+}
+
+int64_t sort_tiles(int64_t n) { return (n + kSortTile - 1) / kSortTile; }
+
+// All launches of one sort on stream s: (k0, v0) sorted by key_bits bits,
+// ping-ponging with (k1, v1); returns the buffer (0 or 1) of the result.
+// counts: kCountWords words; look: sort_look_words(n) words.  ctx (may be
+// null): launch counting and timing.
+int sort_launches(art_ctx* ctx, cudaStream_t s, int sms, uint32_t* k0, uint32_t* v0, uint32_t* k1, uint32_t* v1,
+                  int64_t n, int key_bits, uint32_t* counts, uint32_t* look, unsigned long long* err) {
+  const int64_t nt = sort_tiles(n);
+  const int passes = key_bits / kRadixBits;
+  cudaMemsetAsync(counts, 0, kCountWords * sizeof(uint32_t), s);
+  if (ctx) prof_begin(ctx, "sort_count");
+  radix_count_kernel<<<(unsigned)std::min<int64_t>(nt, 2 * sms), kSortThreads, 0, s>>>(k0, n, passes, counts, look,
+                                                                                       (int64_t)sort_look_words(n));
+  if (ctx) prof_end(ctx);
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)nt);
+  cfg.blockDim = dim3(kSortThreads);
+  cfg.stream = s;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  uint32_t *K[2] = {k0, k1}, *V[2] = {v0, v1};
+  int src = 0;
+  for (int pass = 0; pass < passes; ++pass, src ^= 1) {
+    if (ctx) prof_begin(ctx, "sort_pass");
+    if (n < kSmallSort)
+      cudaLaunchKernelEx(&cfg, radix_pass_kernel<uint32_t>, (const uint32_t*)K[src], (const uint32_t*)V[src], K[src ^ 1],
+                         V[src ^ 1], n, pass, counts, look, err);
+    else
+      cudaLaunchKernelEx(&cfg, radix_pass_kernel<unsigned long long>, (const uint32_t*)K[src], (const uint32_t*)V[src],
+                         K[src ^ 1], V[src ^ 1], n, pass, counts, reinterpret_cast<unsigned long long*>(look), err);
+    if (ctx) prof_end(ctx);
+  }
+  if (ctx) ctx->launches += 1 + passes;
+  return src;
 }
 
 // ---------------------------------------------------- binning by tile buckets
@@ -713,14 +763,12 @@ __global__ void __launch_bounds__(kTileSortThreads) tile_sort_kernel(const uint2
 
 }  // namespace
 
-size_t scan_block_words(int64_t n) { return (size_t)((n + kScanBlock - 1) / kScanBlock) + 1; }
-
 size_t tile_scan_state_words(int64_t ntiles) { return 4 * (size_t)((ntiles + kTileScanBlock - 1) / kTileScanBlock); }
 
-size_t sort_hist_words(int64_t inst_cap) {
-  int64_t nb = (inst_cap + kSortBlock - 1) / kSortBlock;
-  return (size_t)(nb * kRadix);
+size_t sort_look_words(int64_t n) {
+  return (size_t)sort_tiles(n) * kRadix * (n < kSmallSort ? 1 : 2);
 }
+size_t sort_count_words() { return kCountWords; }
 
 void launch_bin(art_ctx* ctx, const ViewParams& v, const uint32_t* hbin, const float* htau, float* thist, bool sort) {
   const int64_t n = ctx->n;
@@ -767,58 +815,30 @@ void launch_bin_views(art_ctx* ctx, const ViewSet& vs, int64_t ntiles) {
              ctx->d_sortlist, nt, vs.v[0].depth_bits, ctx->d_keys, ctx->d_vals, ctx->d_sort_tmp, ctx->d_status);
 }
 
-int launch_sort_bufs(art_ctx* ctx, uint32_t* k0, uint32_t* v0, uint32_t* k1, uint32_t* v1, int64_t cap,
-                     const unsigned long long* count, int key_bits, uint32_t* hist, uint32_t* bsum) {
-  int nb = (int)((cap + kSortBlock - 1) / kSortBlock);
-  if (nb < 1) nb = 1;
-  int64_t hn = (int64_t)nb * kRadix;
-  int hb = (int)((hn + kScanBlock - 1) / kScanBlock);
-  uint32_t* K[2] = {k0, k1};
-  uint32_t* V[2] = {v0, v1};
-  int src = 0;
-  for (int shift = 0; shift < key_bits; shift += kRadixBits) {
-    ART_LAUNCH(ctx, "sort_hist", radix_hist_kernel, nb, kSortThreads, 0, K[src], cap, count, shift, nb, hist);
-    ART_LAUNCH(ctx, "sort_blocksum", block_sum_kernel, hb, kScanThreads, 0, hist, hn,
-               (const unsigned long long*)nullptr, bsum);
-    ART_LAUNCH(ctx, "sort_scan", scan_bsum_kernel, 1, 1024, 0, bsum, hb, (unsigned long long*)nullptr);
-    ART_LAUNCH(ctx, "sort_scanapply", scan_apply_kernel, hb, kScanThreads, 0, hist, hist, hn, bsum);
-    ART_LAUNCH(ctx, "sort_scatter", radix_scatter_kernel, nb, kSortThreads, 0, K[src], V[src], K[src ^ 1],
-               V[src ^ 1], cap, count, shift, nb, hist);
-    src ^= 1;
-  }
-  return src;
-}
-
-namespace {
-__global__ void set_word_kernel(unsigned long long* p, unsigned long long value) { *p = value; }
-}  // namespace
-
-void launch_set_word(art_ctx* ctx, unsigned long long* p, unsigned long long value) {
-  ART_LAUNCH(ctx, "set_word", set_word_kernel, 1, 1, 0, p, value);
+int launch_sort(art_ctx* ctx, uint32_t* k0, uint32_t* v0, uint32_t* k1, uint32_t* v1, int64_t n, int key_bits,
+                uint32_t* counts, uint32_t* look) {
+  return sort_launches(ctx, ctx->stream, ctx->num_sms, k0, v0, k1, v1, n, key_bits, counts, look,
+                       ctx->d_status + kStScanError);
 }
 
 // ------------------------------------------------ sort without allocation
 //
 // art_sort_pairs_static keeps all of its scratch in the fixed device array
 // below instead of memory it allocates: the ping-pong copy of the pairs, the
-// digit histograms, the scan block sums and the key count.  Every kernel of a
-// call rewrites the parts it reads, so nothing carries over from an earlier
-// call and nothing needs clearing.  Calls that overlap on the GPU share the
+// look-back words and the digit counts.  Every call writes the parts it reads
+// first, so nothing carries over from an earlier call.  Calls that overlap on the GPU share the
 // array and race.
 
 namespace {
 
 constexpr int64_t kStaticPairs = ART_SORT_STATIC_MAX_PAIRS;
-constexpr int64_t kStaticBlocks = (kStaticPairs + kSortBlock - 1) / kSortBlock;
-constexpr int64_t kStaticHist = kStaticBlocks * kRadix;
-constexpr int64_t kStaticBsum = (kStaticHist + kScanBlock - 1) / kScanBlock + 1;
 // byte offsets inside the array (each 256-byte aligned)
 constexpr size_t kOffKeys = 0;
 constexpr size_t kOffVals = kOffKeys + 4 * (size_t)kStaticPairs;
-constexpr size_t kOffHist = kOffVals + 4 * (size_t)kStaticPairs;
-constexpr size_t kOffBsum = kOffHist + 4 * (size_t)kStaticHist;
-constexpr size_t kOffCount = (kOffBsum + 4 * (size_t)kStaticBsum + 255) & ~(size_t)255;
-constexpr size_t kStaticBytes = kOffCount + 256;
+constexpr size_t kOffLook = kOffVals + 4 * (size_t)kStaticPairs;
+constexpr size_t kOffCounts = kOffLook + 4 * (size_t)kRadix * ((kStaticPairs + kSortTile - 1) / kSortTile);
+constexpr size_t kStaticBytes = kOffCounts + ((4 * (size_t)kCountWords + 255) & ~(size_t)255);
+static_assert(kStaticPairs < kSmallSort, "32-bit look-back words");
 constexpr int kMaxDevices = 64;
 
 }  // namespace
@@ -912,27 +932,11 @@ extern "C" art_status art_sort_pairs_static(uint32_t* keys, uint32_t* vals, int6
   unsigned char* b = (unsigned char*)base;
   uint32_t* sk = (uint32_t*)(b + kOffKeys);
   uint32_t* sv = (uint32_t*)(b + kOffVals);
-  uint32_t* hist = (uint32_t*)(b + kOffHist);
-  uint32_t* bsum = (uint32_t*)(b + kOffBsum);
-  unsigned long long* count = (unsigned long long*)(b + kOffCount);
-  const int nb = (int)((n + kSortBlock - 1) / kSortBlock);
-  const int64_t hn = (int64_t)nb * kRadix;
-  const int hb = (int)((hn + kScanBlock - 1) / kScanBlock);
-  uint32_t* K[2] = {keys, sk};
-  uint32_t* V[2] = {vals, sv};
-  set_word_kernel<<<1, 1, 0, s>>>(count, (unsigned long long)n);
+  int sms = 0;
+  if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return (cudaGetLastError(), ART_ERR_CUDA);
+  const int src = sort_launches(nullptr, s, sms, keys, vals, sk, sv, n, key_bits, (uint32_t*)(b + kOffCounts),
+                                (uint32_t*)(b + kOffLook), nullptr);
   if (cudaPeekAtLastError() != cudaSuccess) return (cudaGetLastError(), ART_ERR_CUDA);
-  int src = 0;
-  for (int shift = 0; shift < key_bits; shift += kRadixBits) {
-    radix_hist_kernel<<<nb, kSortThreads, 0, s>>>(K[src], n, count, shift, nb, hist);
-    block_sum_kernel<<<hb, kScanThreads, 0, s>>>(hist, hn, nullptr, bsum);
-    scan_bsum_kernel<<<1, 1024, 0, s>>>(bsum, hb, nullptr);
-    scan_apply_kernel<<<hb, kScanThreads, 0, s>>>(hist, hist, hn, bsum);
-    radix_scatter_kernel<<<nb, kSortThreads, 0, s>>>(K[src], V[src], K[src ^ 1], V[src ^ 1], n, count, shift, nb,
-                                                     hist);
-    if (cudaPeekAtLastError() != cudaSuccess) return (cudaGetLastError(), ART_ERR_CUDA);
-    src ^= 1;
-  }
   if (src == 1) {
     if (cudaMemcpyAsync(keys, sk, sizeof(uint32_t) * (size_t)n, cudaMemcpyDeviceToDevice, s) != cudaSuccess ||
         cudaMemcpyAsync(vals, sv, sizeof(uint32_t) * (size_t)n, cudaMemcpyDeviceToDevice, s) != cudaSuccess)

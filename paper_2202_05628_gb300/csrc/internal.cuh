@@ -42,7 +42,7 @@ enum StatusWord {
   kStSortBig = 16,      // binning: buckets sorted by a whole block
   kStSortBigNext = 17,  // binning: next such bucket (work counter)
   kStScanTicket = 18,   // binning: blocks of the tile scan started (their order)
-  kStScanError = 19,    // binning: tile-scan blocks that timed out waiting for a predecessor
+  kStScanError = 19,    // binning, sort: look-backs that timed out waiting for a predecessor
   kStActiveGroups = 20, // binning: groups of four consecutive tiles with instances (listed in d_agroups)
   kStExactQ = 21,       // composite: tiles queued for the exact re-walk (a pixel's reorder buffer overflowed)
   kStGridCells = 22,    // lattice index: occupied cells of the last pose
@@ -274,8 +274,8 @@ struct art_ctx {
   // ---- art_sort_pairs scratch
   uint32_t* d_sk = nullptr;
   uint32_t* d_sv = nullptr;
-  uint32_t* d_shist = nullptr;
-  uint32_t* d_sbsum = nullptr;
+  uint32_t* d_slook = nullptr;
+  uint32_t* d_scounts = nullptr;
   int64_t sort_cap = 0;
 
   // ---- profiling
@@ -335,13 +335,13 @@ void launch_tile_sort(art_ctx* ctx, const ViewParams& v);
 // depth_bits): one scan of all tiles' counts, one scatter per view (its
 // instances keyed by global tile), one sort of all buckets.
 void launch_bin_views(art_ctx* ctx, const ViewSet& vs, int64_t ntiles);
-// Radix sort of count (device word) pairs ping-ponging between (k0, v0) and
-// (k1, v1); returns the index (0 or 1) of the buffer holding the result.
-int launch_sort_bufs(art_ctx* ctx, uint32_t* k0, uint32_t* v0, uint32_t* k1, uint32_t* v1, int64_t cap,
-                     const unsigned long long* count, int key_bits, uint32_t* hist, uint32_t* bsum);
-void launch_set_word(art_ctx* ctx, unsigned long long* p, unsigned long long value);
-size_t sort_hist_words(int64_t n);
-size_t scan_block_words(int64_t n);
+// Radix sort of n pairs ping-ponging between (k0, v0) and (k1, v1); returns
+// the index (0 or 1) of the buffer holding the result.  counts and look: scratch
+// of sort_count_words() and sort_look_words(n) words.
+int launch_sort(art_ctx* ctx, uint32_t* k0, uint32_t* v0, uint32_t* k1, uint32_t* v1, int64_t n, int key_bits,
+                uint32_t* counts, uint32_t* look);
+size_t sort_look_words(int64_t n);
+size_t sort_count_words();
 size_t tile_scan_state_words(int64_t ntiles);  // look-back words of the tile scan
 
 // ---- depth buffer (depth.cu): after launch_project + launch_bin of the view,
