@@ -288,7 +288,9 @@ art_status ensure_skip_buffers(art_ctx* ctx, const ViewParams& v) {
 art_status ensure_split_buffers(art_ctx* ctx, size_t ntiles) {
   art_status st;
   // a tile of len entries is cut into ceil(len / seg_len) <= len / seg_len + 1 segments
-  const size_t items = (size_t)(ctx->inst_cap / std::max(32, ctx->seg_len)) + ntiles + 1;
+  // (shorter default segments: at most one per resident walk warp more, seg_plan_kernel)
+  const size_t items =
+      (size_t)(ctx->inst_cap / std::max(32, ctx->seg_len)) + 2 * (size_t)ctx->num_sms * kMaxWalkBlocks + ntiles + 1;
   if ((st = ensure(ctx, (void**)&ctx->d_seg, &ctx->d_seg_bytes, ntiles * sizeof(uint2), "segment plan")) != ART_OK)
     return st;
   if ((st = ensure(ctx, (void**)&ctx->d_multi, &ctx->d_multi_bytes, ntiles * 4, "split tiles")) != ART_OK) return st;
@@ -827,7 +829,7 @@ art_status art_load_sh_features(art_ctx* ctx, int degree, const float* coef) {
   const size_t count = (size_t)ctx->n * (size_t)((degree + 1) * (degree + 1)) * (size_t)ctx->C;
   art_status st;
   if ((st = alloc(ctx, &ctx->d_sh, count, "SH coefficients")) != ART_OK) return st;
-  if ((st = alloc(ctx, &ctx->d_sh_rot, 9 * (size_t)ctx->n, "SH rotations")) != ART_OK) return st;
+  if ((st = alloc(ctx, &ctx->d_sh_rot, 3 * (size_t)ctx->n, "SH rotations")) != ART_OK) return st;
   cudaError_t e = cudaMemcpyAsync(ctx->d_sh, coef, sizeof(float) * count, cudaMemcpyDefault, ctx->stream);
   if (e != cudaSuccess) return cuda_fail(ctx, e, "copy SH coefficients");
   if ((st = sync_check(ctx, "load_sh_features")) != ART_OK) return st;

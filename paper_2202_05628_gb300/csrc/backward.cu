@@ -250,11 +250,7 @@ __global__ void __launch_bounds__(32) bwd_split_kernel(
   const int lane = threadIdx.x & 31;
   const unsigned long long n_items = status[kStItems];
   const uint32_t wq = seg_window(v, status);
-  for (;;) {
-    unsigned long long i = 0;
-    if (lane == 0) i = atomicAdd(status + kStNext, 1ull);
-    i = __shfl_sync(0xffffffffu, i, 0);
-    if (i >= n_items) break;
+  for (unsigned long long i = blockIdx.x; i < n_items; i = next_item(status, n_items, lane)) {
     const int tile = (int)items[i];
     const uint2 sgt = seg[tile];
     if (PASS == 0 && sgt.y < 2) continue;
@@ -358,9 +354,11 @@ void launch_bwd_c(art_ctx* ctx, const ViewParams& v, const float* F, const float
                   const float* dA, float* gfeat, float* gsig) {
   const int ntiles = v.tiles_x * v.tiles_y;
   const TF* feat = (const TF*)ctx->d_feat;
-  cudaMemsetAsync(ctx->d_status + kStItems, 0, 4 * sizeof(unsigned long long), ctx->stream);  // items .. next merge
+  cudaMemsetAsync(ctx->d_status + kStItems, 0, 4 * sizeof(unsigned long long), ctx->stream);  // items .. the walk's counter
+  // (a length other than the default is the caller's)
+  const int walkers = ctx->seg_len == kSegDefault ? ctx->composite_blocks : 0;
   ART_LAUNCH(ctx, "composite_plan", seg_plan_kernel, (ntiles + 255) / 256, 256, 0, ntiles, ctx->d_ranges,
-             ctx->seg_len, ctx->d_seg, ctx->d_items, ctx->d_multi, ctx->d_status, (const uint32_t*)nullptr, 0);
+             ctx->seg_len, walkers, ctx->d_seg, ctx->d_items, ctx->d_multi, ctx->d_status);
   const int grid = ctx->composite_blocks;
   auto k0 = bwd_split_kernel<C, TF, 0>;
   ART_LAUNCH(ctx, "composite_bwd_scan", k0, grid, 32, 0, ctx->d_ranges, ctx->d_seg, ctx->d_items, ctx->d_keys,

@@ -47,7 +47,7 @@ __device__ uint32_t block_exclusive_scan(uint32_t v, uint32_t* total) {
 // Stable LSD radix sort of 32-bit pairs, eight bits a pass: one kernel counts
 // every pass's digits over all keys, then one kernel per pass ranks, exchanges
 // and scatters.  A block takes the next tile of 4096 pairs (a ticket, so every
-// predecessor is running), ranks its pairs by warp matches, publishes its digit
+// predecessor is running), ranks its pairs by warp ballots, publishes its digit
 // counts, and thread d looks back over the earlier tiles' counts of digit d,
 // sixteen of them per round: all of a small sort's tiles run at once, so the
 // nearest published prefix is far at first and a walk one tile at a time would
@@ -147,8 +147,15 @@ __global__ void __launch_bounds__(kSortThreads) radix_pass_kernel(const uint32_t
 #pragma unroll
   for (int r = 0; r < kSortRounds; ++r) {
     const bool in = w * (32 * kSortRounds) + r * 32 + lane < m;
-    const uint32_t d = in ? (key[r] >> shift) & (kRadix - 1) : (uint32_t)kRadix;
-    const unsigned peers = __match_any_sync(0xffffffffu, d);
+    const uint32_t d = (key[r] >> shift) & (kRadix - 1);
+    // the lanes with this digit, by eight ballots (a match of many different values takes ~60 cycles of the SM)
+    unsigned peers = __ballot_sync(0xffffffffu, in);
+#pragma unroll
+    for (int b = 0; b < kRadixBits; ++b) {
+      const bool one = (d >> b) & 1u;
+      const unsigned ones = __ballot_sync(0xffffffffu, one);
+      peers &= one ? ones : ~ones;
+    }
     const int leader = __ffs(peers) - 1;
     uint32_t before = 0;
     if (in && lane == leader) {
@@ -156,7 +163,7 @@ __global__ void __launch_bounds__(kSortThreads) radix_pass_kernel(const uint32_t
       wh[w][d] = before + __popc(peers);
     }
     __syncwarp();
-    rank[r] = __shfl_sync(0xffffffffu, before, leader) + __popc(peers & lt);
+    rank[r] = __shfl_sync(0xffffffffu, before, leader & 31) + __popc(peers & lt);
   }
   __syncthreads();
   // thread t = digit t: offsets of the warps, the tile's count, published
@@ -284,7 +291,7 @@ constexpr int kSortPer = 16;             // bucket entries per thread held in re
 constexpr int kSortRegs = kTileSortThreads * kSortPer;  // buckets held in registers (8192)
 constexpr int kTileSortSmem = kSortRegs;                 // ... and staged in shared memory (64 KB)
 constexpr int kWarpSortCap = 256;        // buckets up to this size: one warp each
-constexpr int kSortBins = 4096;          // depth bins of a block-sorted bucket
+constexpr int kSortBins = 4096;          // depth bins of a block-sorted bucket (512 for short buckets measured 2 us slower)
 constexpr int kRankMax = 64;             // bins up to this size: entries ranked by counting
 
 // The tiles x0..x1 by y0..y1 of a pixel rectangle, the k-th in row-major order.
@@ -306,7 +313,7 @@ __device__ __forceinline__ uint32_t rect_tile(const ViewParams& v, int tx0, int 
 // total into kStInstances, and the tiles whose bucket needs sorting: those of
 // 2..kWarpSortCap instances from the front of sort_list, longer ones from its
 // end (kStSortTiles and kStSortBig of them, written by the last block, which
-// also resets both work counters).  The counts it reads are zeroed for the
+// also resets the block-sorted ones' work counter).  The counts it reads are zeroed for the
 // next projection, and with thist the 64 depth bins of every tile with
 // instances are zeroed for the scatter that adds into them (rows of tiles
 // without instances are not read).
@@ -475,7 +482,6 @@ __global__ void __launch_bounds__(kTileScanThreads) tile_scan_kernel(int ntiles,
     status[kStInstances] = pi + tot;
     status[kStSortTiles] = (pl & 0x7FFFFFFFull) + (lt & 0xFFFFu);
     status[kStSortBig] = (pl >> 31) + (lt >> 16);
-    status[kStSortNext] = 0;
     status[kStSortBigNext] = 0;
   }
 }
@@ -551,31 +557,29 @@ __global__ void __launch_bounds__(256) bucket_emit_kernel(int64_t n, const uint3
 // +infinity and are never touched, so any n works.  Lanes t0, t0 + 32, ...
 // of one warp share the comparators of s[0, n).
 __device__ void warp_bitonic(unsigned long long* s, uint32_t n, uint32_t t0) {
-  uint32_t P = 1;
-  while (P < n) P <<= 1;
-  for (uint32_t k = 2; k <= P; k <<= 1) {
-    const uint32_t half = k >> 1;
-    for (uint32_t i = t0; i < P / 2; i += 32) {  // merge: mirrored pairs
-      const uint32_t a = (i / half) * k + i % half, b = (i / half) * k + k - 1 - i % half;
-      if (b < n) {
-        const unsigned long long x = s[a], y = s[b];
-        if (y < x) {
-          s[a] = y;
-          s[b] = x;
-        }
+  uint32_t lp = 0;  // 2^lp >= n
+  while ((1u << lp) < n) ++lp;
+  const uint32_t pairs = (1u << lp) / 2;
+  // (positions by shifts: run-time divisions made a 256-entry sort ~10 us)
+  auto exchange = [&](uint32_t a, uint32_t b) {
+    if (b < n) {
+      const unsigned long long x = s[a], y = s[b];
+      if (y < x) {
+        s[a] = y;
+        s[b] = x;
       }
     }
+  };
+  for (uint32_t l = 1; l <= lp; ++l) {
+    for (uint32_t i = t0; i < pairs; i += 32) {  // merge of runs of 2^l: mirrored pairs
+      const uint32_t g = (i >> (l - 1)) << l, r = i & ((1u << (l - 1)) - 1u);
+      exchange(g + r, g + (1u << l) - 1u - r);
+    }
     __syncwarp();
-    for (uint32_t j = k >> 2; j > 0; j >>= 1) {  // half-cleaners
-      for (uint32_t i = t0; i < P / 2; i += 32) {
-        const uint32_t a = (i / j) * 2 * j + i % j, b = a + j;
-        if (b < n) {
-          const unsigned long long x = s[a], y = s[b];
-          if (y < x) {
-            s[a] = y;
-            s[b] = x;
-          }
-        }
+    for (uint32_t m = l - 1; m-- > 0;) {  // half-cleaners at distance 2^m
+      for (uint32_t i = t0; i < pairs; i += 32) {
+        const uint32_t a = ((i >> m) << (m + 1)) + (i & ((1u << m) - 1u));
+        exchange(a, a + (1u << m));
       }
       __syncwarp();
     }
@@ -712,7 +716,9 @@ __device__ void block_sort_bucket(uint32_t* __restrict__ keys, uint32_t* __restr
 
 // Sort each listed tile's bucket by (depth quantum, voxel id).  Persistent
 // blocks take the buckets of more than kWarpSortCap entries first, one block
-// each, then the others, one warp each.
+// each (the first by block index, further ones from a counter), then the
+// others, one warp each in turn.  (Counters for both cost ~10 us even on frames
+// with few buckets: one atomic of every warp on one word.)
 __global__ void __launch_bounds__(kTileSortThreads) tile_sort_kernel(const uint2* __restrict__ ranges,
                                                                      const uint32_t* __restrict__ sort_list,
                                                                      int ntiles, int depth_bits,
@@ -725,26 +731,23 @@ __global__ void __launch_bounds__(kTileSortThreads) tile_sort_kernel(const uint2
   __shared__ unsigned long long s_item;
   const uint32_t qmask = (1u << depth_bits) - 1u;
   const unsigned long long n_big = status[kStSortBig], n_small = status[kStSortTiles];
-  for (;;) {
-    if (threadIdx.x == 0) s_item = atomicAdd(status + kStSortBigNext, 1ull);
-    __syncthreads();
-    const unsigned long long it = s_item;
-    __syncthreads();
-    if (it >= n_big) break;
+  for (unsigned long long it = blockIdx.x; it < n_big;) {
     const uint32_t tile = sort_list[ntiles - 1 - (int)it];
     const uint2 rg = ranges[tile];
     const uint32_t n = rg.y - rg.x;
     if (n > 1)
       block_sort_bucket(keys + rg.x, vals + rg.x, n, qmask, tile << depth_bits,
                         n <= (uint32_t)kTileSortSmem ? sk : scratch + rg.x);
+    if (n_big <= gridDim.x) break;
+    if (threadIdx.x == 0) s_item = gridDim.x + atomicAdd(status + kStSortBigNext, 1ull);
+    __syncthreads();
+    it = s_item;
+    __syncthreads();
   }
   const uint32_t lane = threadIdx.x & 31u;
   unsigned long long* ws = sk + (threadIdx.x >> 5) * kWarpSortCap;
-  for (;;) {
-    unsigned long long it = 0;
-    if (lane == 0) it = atomicAdd(status + kStSortNext, 1ull);
-    it = __shfl_sync(0xFFFFFFFFu, it, 0);
-    if (it >= n_small) break;
+  for (unsigned long long it = (unsigned long long)(threadIdx.x >> 5) * gridDim.x + blockIdx.x; it < n_small;
+       it += (unsigned long long)kTileSortWarps * gridDim.x) {
     const uint32_t tile = sort_list[it];
     const uint2 rg = ranges[tile];
     const uint32_t n = rg.y - rg.x;

@@ -18,6 +18,9 @@ namespace art {
 
 constexpr int kMaxJoints = 64;
 constexpr int kMaxViews = 8;
+constexpr int kMaxWalkBlocks = 12;  // one-warp blocks of the composite walk per SM, at most
+constexpr int kSegDefault = 256;  // default list entries per composite segment
+constexpr int kSegShortest = 64;  // ... of the backward, where a view has too few for the GPU
 constexpr int kOpacityPad = 32;  // two-branch network: channels of the opacity branch's packed input [A, I_f, 0 ...]
 constexpr float kDetMin = 1e-3f;   // blended transforms below this are dropped
 constexpr float kZMin = 1e-6f;     // corners must lie in front of the camera
@@ -33,14 +36,14 @@ enum StatusWord {
   kStFallback = 5,      // tiles queued for the full traversal (last render)
   kStItems = 8,         // composite segments planned (last render)
   kStMulti = 9,         // tiles split into two or more segments
-  kStNext = 10,         // next segment to walk (work counter)
-  kStNextMerge = 11,    // next split tile to merge (work counter)
+  kStNext = 10,         // segments taken beyond each block's first (work counter)
+  kStReserved11 = 11,   // (reserved)
   kStRmax = 12,         // largest voxel bounding radius of the last pose (float bits)
   kStReserved13 = 13,   // (reserved)
   kStSortTiles = 14,    // binning: tiles whose bucket needs sorting
-  kStSortNext = 15,     // binning: next bucket to sort (work counter)
+  kStReserved15 = 15,   // (reserved)
   kStSortBig = 16,      // binning: buckets sorted by a whole block
-  kStSortBigNext = 17,  // binning: next such bucket (work counter)
+  kStSortBigNext = 17,  // binning: such buckets taken beyond each block's first (work counter)
   kStScanTicket = 18,   // binning: blocks of the tile scan started (their order)
   kStScanError = 19,    // binning, sort: look-backs that timed out waiting for a predecessor
   kStActiveGroups = 20, // binning: groups of four consecutive tiles with instances (listed in d_agroups)
@@ -197,7 +200,7 @@ struct art_ctx {
   unsigned long long* d_status = nullptr;
   unsigned long long* h_status = nullptr;  // pinned
   float* d_sh = nullptr;        // [n][(L+1)^2][C] spherical-harmonics coefficients (view-dependent features)
-  float* d_sh_rot = nullptr;    // [n][9] world -> canonical direction map per voxel
+  float4* d_sh_rot = nullptr;   // [n][3] rows (xyz) of the world -> canonical direction map per voxel
   int sh_degree = -1;           // L, or -1: plain features
   bool attr_tile_sort = false;  // large shared-memory attributes set on this context's device
   bool attr_proposal = false;
@@ -256,7 +259,7 @@ struct art_ctx {
   float2* d_xhit = nullptr;       // [blocks][32][kExactCap] per-lane hit lists (t0, chord) ...
   uint32_t* d_xpos = nullptr;     // ... and list positions
   // ---- split composite walk
-  int seg_len = 256;              // list entries per segment
+  int seg_len = art::kSegDefault;  // list entries per segment
   int composite_blocks = 0;       // persistent one-warp blocks of the split walk
   int composite_key = 0;          // (C, feature bytes) composite_blocks was computed for
   uint2* d_seg = nullptr;         // [tiles] (first segment, segment count)

@@ -139,7 +139,7 @@ constexpr int NT = 32;           // instances per staged chunk
 
 // Resident one-warp blocks of the composite walk per SM (its register cap is
 // 64K / (32 x this)) and the shared memory of each block's feature ring.
-constexpr int kCompositeWarps = 12;
+constexpr int kCompositeWarps = kMaxWalkBlocks;
 constexpr int kRingBytes = 10240;
 
 template <int C, typename TF>
@@ -408,19 +408,19 @@ constexpr int kMaxSegs = 255;
 
 // Per tile: number of segments and the index of its first one; the segments
 // of all tiles in one list, the tiles with two or more in another.
-// With tiles_in set, only the tiles listed there (count in status[in_word]).
-static __global__ void seg_plan_kernel(int ntiles, const uint2* __restrict__ ranges, int seg_len, uint2* __restrict__ seg,
-                                uint32_t* __restrict__ items, uint32_t* __restrict__ multi,
-                                unsigned long long* __restrict__ status, const uint32_t* __restrict__ tiles_in,
-                                int in_word) {
+// With walkers set (the resident warps), segments are as short as gives every
+// warp one, down to kSegShortest.  The backward does: a view of few instances
+// is bound by its longest segment's walk.  The composite keeps its length, so
+// that a map's rounding depends on the tile alone, not on the frame's instances.
+static __global__ void seg_plan_kernel(int ntiles, const uint2* __restrict__ ranges, int seg_len, int walkers,
+                                       uint2* __restrict__ seg, uint32_t* __restrict__ items,
+                                       uint32_t* __restrict__ multi, unsigned long long* __restrict__ status) {
   ART_PDL_ENTRY();
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  int t = i;
-  if (tiles_in) {
-    if ((unsigned long long)i >= status[in_word]) return;
-    t = (int)tiles_in[i];
-  }
+  const int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= ntiles) return;
+  if (walkers > 0)
+    seg_len = (int)min((unsigned long long)seg_len,
+                       max((unsigned long long)kSegShortest, status[kStInstances] / (unsigned)walkers));
   const uint2 rg = ranges[t];
   const uint32_t len = rg.y - rg.x;
   uint32_t S = len == 0 ? 0u : (len + seg_len - 1) / seg_len;
@@ -432,6 +432,15 @@ static __global__ void seg_plan_kernel(int ntiles, const uint2* __restrict__ ran
     if (S > 1) multi[atomicAdd(status + kStMulti, 1ull)] = (uint32_t)t;
   }
   seg[t] = make_uint2(base, S);
+}
+
+// The segment a persistent one-warp block walks after its first (segment
+// blockIdx.x): from a counter, so that blocks with short segments take more.
+__device__ __forceinline__ unsigned long long next_item(unsigned long long* status, unsigned long long n_items, int lane) {
+  if (n_items <= gridDim.x) return n_items;
+  unsigned long long i = 0;
+  if (lane == 0) i = gridDim.x + atomicAdd(status + kStNext, 1ull);
+  return __shfl_sync(0xffffffffu, i, 0);
 }
 
 // First position in [a, b) whose depth quantum is >= qt (b if none): keys are
