@@ -20,7 +20,7 @@
 // column phases px x 32 output channels of one output row 2i + py (one TMEM
 // accumulator of 64 columns), K = taps x channels.  A CTA computes one row
 // phase py (blockIdx parity) for all its units, so it keeps only that
-// phase's weight blocks resident (68 KB for the 96 -> 32 layer) and two CTAs
+// phase's weight blocks resident (50 KB for the 96 -> 32 layer) and two CTAs
 // share an SM: two threads issue MMAs there.  A stage is one TMA box of 130
 // pixels (j0 - 1 .. j0 + 128) x 32 channels of one input row: of u (rows
 // i + oy, oy in {py - 1, py}), or of s (rows 2i + r, r in {py - 1, py,
@@ -52,6 +52,7 @@ constexpr int kBoxBytes = kHalo * kKCB;
 constexpr int kStageBytes = (kBoxBytes + 511) / 512 * 512;  // stages on 64-B swizzle atoms (8 rows x 64 B)
 constexpr int kBlock = kC * kKCB;  // one weight block: 32 output x 32 input channels
 constexpr int kSkipEntries = 18;   // per row phase: (r, c, px) of the skip part
+constexpr int kSkipBlocks = 9;     // ... of which nine differ: (dy, dx), kept in shared memory
 constexpr int kUpEntries = 8;      // per row phase: (oy, ox, px) of the low-resolution part
 constexpr int kAccCols = 2 * kC;   // one accumulator: two column phases x 32 channels
 constexpr int kMaxWeights = 80 * 1024;
@@ -66,20 +67,27 @@ __host__ __device__ constexpr int skip_min(int v) { return v == 2 ? 1 : 0; }
 // (ox = -1, 0) and px = 1 (ox = 0, 1).
 __host__ __device__ constexpr int up_n(int v) { return v == 0 ? 2 : 1; }
 __host__ __device__ constexpr int up_min(int v) { return v == 1 ? 1 : 0; }
-// First weight block of column offset c among one input row's six skip
-// entries (ordered by c, then px; the rows r = py - 1 .. py + 1 follow each
-// other), of ox among one low-resolution row's four (rows oy = py - 1, py).
-__host__ __device__ constexpr int skip_block(int c) {
+// The skip part's weights do not depend on the phase, so an input row needs its
+// three taps' blocks once, in the order dx = 1, 0, -1: column phases 0 and 1
+// then find theirs side by side (c = 0: dx = 0, -1; c = 1: dx = 1, 0).  First
+// block of column offset c; the rows r = py - 1 .. py + 1 follow each other.
+__host__ __device__ constexpr int skip_block(int c) { return 1 - (c - skip_min(c)); }
+// First weight entry of column offset c among one input row's six in the
+// weights' global layout (ordered by c, then px).
+__host__ __device__ constexpr int skip_entry(int c) {
   int b = 0;
   for (int cc = -1; cc < c; ++cc) b += skip_n(cc);
   return b;
 }
+// First weight block of ox among one low-resolution row's four (ordered by ox,
+// then px; rows oy = py - 1, py).
 __host__ __device__ constexpr int up_block(int ox) {
   int b = 0;
   for (int xx = -1; xx < ox; ++xx) b += up_n(xx);
   return b;
 }
-static_assert(3 * (skip_block(2) + 1) == kSkipEntries && 2 * (up_block(1) + 1) == kUpEntries, "entry tables");
+static_assert(3 * (skip_entry(2) + 1) == kSkipEntries && 2 * (up_block(1) + 1) == kUpEntries, "entry tables");
+static_assert(skip_block(0) == 1 && skip_block(1) == 0 && skip_block(-1) == 2 && skip_block(2) == 0, "block order");
 
 // floor(v / 2) for v in {-1, 0, 1, 2}
 __host__ __device__ constexpr int half_floor(int v) { return (v + 2) / 2 - 1; }
@@ -98,12 +106,11 @@ struct SubParams {
 // MMA of one column offset whose column phases are px0 .. px0 + nc - 1
 // (TMEM columns and weight blocks consecutive).  Two K steps of 16
 // channels each.
-__device__ __forceinline__ void sub_mma(uint32_t d, uint32_t a, uint32_t wb0, int nc, int px0) {
+__device__ __forceinline__ void sub_mma(uint32_t d, uint64_t a, uint64_t w, int nc, int px0) {
   const uint32_t idesc = nc == 2 ? idesc_bf16(128, 2 * kC) : idesc_bf16(128, kC);
   const uint32_t dc = d + (uint32_t)(px0 * kC);
 #pragma unroll
-  for (int kk = 0; kk < kKCB / 32; ++kk)
-    umma<false>(dc, umma_desc<kKCB>(a + kk * 32), umma_desc<kKCB>(wb0 + kk * 32), idesc, 1u);
+  for (int kk = 0; kk < kKCB / 32; ++kk) umma<false>(dc, a + kk * 2, w + kk * 2, idesc, 1u);
 }
 
 __global__ void __launch_bounds__(kThreads, kCtas)
@@ -112,7 +119,7 @@ __global__ void __launch_bounds__(kThreads, kCtas)
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
   uint8_t* sm = smem_raw + (((raw + 1023u) & ~1023u) - raw);
-  uint8_t* wsm = sm;  // row phase py's skip blocks [cs_ch][18], then low-resolution blocks [cu_ch][8], 2 KB each
+  uint8_t* wsm = sm;  // skip blocks [cs_ch][9], then row phase py's low-resolution blocks [cu_ch][8], 2 KB each
   uint8_t* stages = sm + p.w_bytes;
   const int S = p.n_stages;
   uint64_t* full = reinterpret_cast<uint64_t*>(stages + (size_t)S * kStageBytes);
@@ -129,7 +136,7 @@ __global__ void __launch_bounds__(kThreads, kCtas)
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int py = blockIdx.x & 1;                  // this CTA's output rows 2i + py
   const int u0 = blockIdx.x >> 1, du = gridDim.x >> 1;
-  const int ubase_off = p.cs_ch * kSkipEntries * kBlock;
+  const int ubase_off = p.cs_ch * kSkipBlocks * kBlock;
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < S; ++s) {
@@ -157,9 +164,9 @@ __global__ void __launch_bounds__(kThreads, kCtas)
     if (lane == 0) {
       mbar_expect_tx(wbar, (uint32_t)p.w_bytes);  // the weights are static: loaded before the wait
       for (int cc = 0; cc < p.cs_ch; ++cc)
-        for (int e = 0; e < kSkipEntries; ++e)
-          tma_load_2d(wsm + (size_t)(cc * kSkipEntries + e) * kBlock, &tmWs, wbar, cc * kKC,
-                      (py * kSkipEntries + e) * kC);
+        for (int b = 0; b < kSkipBlocks; ++b)  // tap (b / 3 - 1, 1 - b % 3): column phase 0's entry at c = dx
+          tma_load_2d(wsm + (size_t)(cc * kSkipBlocks + b) * kBlock, &tmWs, wbar, cc * kKC,
+                      (py * kSkipEntries + 6 * (b / 3) + skip_entry(1 - b % 3)) * kC);
       for (int cc = 0; cc < p.cu_ch; ++cc)
         for (int e = 0; e < kUpEntries; ++e)
           tma_load_2d(wsm + ubase_off + (size_t)(cc * kUpEntries + e) * kBlock, &tmWu, wbar, cc * kKC,
@@ -212,12 +219,14 @@ __global__ void __launch_bounds__(kThreads, kCtas)
       int s = 0, buf = 0;
       uint32_t ph = 0, aph = 0;
       bool ok = mbar_wait(wbar, 0u, abort_flag);
-      const uint32_t wbase = smem_u32(wsm), ubase = wbase + (uint32_t)ubase_off;
-      uint32_t a0 = 0;  // the stage in hand
+      // operand descriptors advance by constants (rebuilt per MMA they held its issue at ~130 cycles)
+      const uint64_t wbase = umma_desc<kKCB>(smem_u32(wsm)), ubase = wbase + (uint32_t)(ubase_off >> 4);
+      const uint64_t abase = umma_desc<kKCB>(smem_u32(stages));
+      uint64_t a0 = 0;  // the stage in hand
       auto next_full = [&]() {
         if (!mbar_wait(&full[s], ph, abort_flag)) return false;
         tc_fence_after();
-        a0 = smem_u32(stages + (size_t)s * kStageBytes);
+        a0 = abase + (uint32_t)(s * (kStageBytes >> 4));
         return true;
       };
       auto release = [&]() {
@@ -232,24 +241,25 @@ __global__ void __launch_bounds__(kThreads, kCtas)
         if (!mbar_wait(&acce[buf], aph, abort_flag)) break;
         tc_fence_after();
         const uint32_t d0 = tmem_base + (uint32_t)(buf * kAccCols);
-        uint32_t wb = wbase;  // weight blocks of the (chunk, row) in hand
+        uint64_t wb = wbase;  // weight blocks of the (chunk, row) in hand
+        constexpr uint64_t kRow = kKCB >> 4, kB = kBlock >> 4;
         // even box: c = 0 (from row 1), c = 2 (row 2); odd box: c = -1 (row 0), c = 1 (row 1)
-        for (int cr = 0; ok && cr < 3 * p.cs_ch; ++cr, wb += 6 * kBlock) {
+        for (int cr = 0; ok && cr < 3 * p.cs_ch; ++cr, wb += 3 * kB) {
           if (!(ok = next_full())) break;
-          sub_mma(d0, a0 + 1 * kKCB, wb + skip_block(0) * kBlock, skip_n(0), skip_min(0));
-          sub_mma(d0, a0 + 2 * kKCB, wb + skip_block(2) * kBlock, skip_n(2), skip_min(2));
+          sub_mma(d0, a0 + 1 * kRow, wb + skip_block(0) * kB, skip_n(0), skip_min(0));
+          sub_mma(d0, a0 + 2 * kRow, wb + skip_block(2) * kB, skip_n(2), skip_min(2));
           release();
           if (!(ok = next_full())) break;
-          sub_mma(d0, a0 + 0 * kKCB, wb + skip_block(-1) * kBlock, skip_n(-1), skip_min(-1));
-          sub_mma(d0, a0 + 1 * kKCB, wb + skip_block(1) * kBlock, skip_n(1), skip_min(1));
+          sub_mma(d0, a0 + 0 * kRow, wb + skip_block(-1) * kB, skip_n(-1), skip_min(-1));
+          sub_mma(d0, a0 + 1 * kRow, wb + skip_block(1) * kB, skip_n(1), skip_min(1));
           release();
         }
         wb = ubase;
-        for (int co = 0; ok && co < 2 * p.cu_ch; ++co, wb += 4 * kBlock) {
+        for (int co = 0; ok && co < 2 * p.cu_ch; ++co, wb += 4 * kB) {
           if (!(ok = next_full())) break;
 #pragma unroll
           for (int ox = -1; ox <= 1; ++ox)
-            sub_mma(d0, a0 + (uint32_t)((ox + 1) * kKCB), wb + up_block(ox) * kBlock, up_n(ox), up_min(ox));
+            sub_mma(d0, a0 + (uint64_t)(ox + 1) * kRow, wb + up_block(ox) * kB, up_n(ox), up_min(ox));
           release();
         }
         if (!ok) break;
@@ -471,7 +481,7 @@ art_status launch_sub_conv(art_ctx* ctx, const SubConv& c) {
   p.cu_ch = c.cu / kKC;
   p.tiles_per_row = (w + 127) / 128;
   p.n_units = p.tiles_per_row * h;
-  p.w_bytes = (kSkipEntries * p.cs_ch + kUpEntries * p.cu_ch) * kBlock;
+  p.w_bytes = (kSkipBlocks * p.cs_ch + kUpEntries * p.cu_ch) * kBlock;
   p.bias = c.bias;
   p.out = (__nv_bfloat16*)c.out;
   p.err = ctx->d_status + kStTcError;

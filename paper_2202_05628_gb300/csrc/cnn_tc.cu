@@ -533,6 +533,7 @@ __global__ void __launch_bounds__(kThreads, TcCfg<N, KCB, F8>::kCtas)
     if (lane == 0) {
       int s = 0, buf = 0;
       uint32_t ph = 0, aph = 0;
+      const uint64_t a_desc = umma_desc<KCB>(smem_u32(stages));  // descriptors advance by constants
       for (int tile = blockIdx.x; tile < p.n_tiles && !*abort_flag; tile += gridDim.x) {
         if (!mbar_wait(&acce[buf], aph ^ 1u, abort_flag)) break;
         tc_fence_after();
@@ -544,10 +545,10 @@ __global__ void __launch_bounds__(kThreads, TcCfg<N, KCB, F8>::kCtas)
             break;
           }
           tc_fence_after();
-          const uint32_t a = smem_u32(stages + s * Cfg::kStage), b = a + Cfg::kA;
+          const uint64_t a = a_desc + (uint32_t)(s * (Cfg::kStage >> 4));
 #pragma unroll
           for (int kk = 0; kk < KCB / 32; ++kk)
-            umma<F8>(d, umma_desc<KCB>(a + kk * 32), umma_desc<KCB>(b + kk * 32), Cfg::kIdesc, (c | kk) != 0);
+            umma<F8>(d, a + kk * 2, a + (Cfg::kA >> 4) + kk * 2, Cfg::kIdesc, (c | kk) != 0);
           umma_commit(&empty[s]);
           if (++s == Cfg::kStages) {
             s = 0;
@@ -611,6 +612,8 @@ __global__ void __launch_bounds__(kThreads, TcCfg<N, KCB, F8>::kCtas)
 // 9, and no weight traffic.  Accumulators: R x N TMEM columns per unit, two
 // units in flight.
 constexpr int kRows = 4;
+constexpr int kRowEpiWarps = 8;
+constexpr int kRowThreads = 64 + 32 * kRowEpiWarps;  // warp 0 TMA, warp 1 MMA + TMEM, warps 2..9 epilogue
 
 // The vertical taps are stacked into one operand:
 // the accumulators of the unit's R output rows sit in consecutive TMEM
@@ -625,6 +628,7 @@ struct RowCfg {
   static constexpr int kSlots = kRows;
   static constexpr int kBufCols = kSlots * N;  // columns of one accumulator buffer
   static constexpr int kHalo = 130;                                   // input pixels of a row box (128 + 2)
+  static constexpr int kMinCtas = N * KCB >= 64 * 128 && !F8 ? 1 : 2;  // (the widest one's weights leave room for one)
   // one input row per stage; two measured slower on the 32-channel layers
   // (a deeper box per barrier round trip, half as many stages in flight)
   static constexpr int kBoxBytes = kHalo * KCB;
@@ -641,7 +645,7 @@ struct RowParams {
 };
 
 template <int N, int KCB, bool F8>
-__global__ void __launch_bounds__(kThreads, 2)
+__global__ void __launch_bounds__(kRowThreads, (RowCfg<N, KCB, F8>::kMinCtas))
     conv_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, RowParams rp) {
   using Cfg = RowCfg<N, KCB, F8>;
   const TcParams& p = rp.p;
@@ -680,18 +684,18 @@ __global__ void __launch_bounds__(kThreads, 2)
     }
     for (int b = 0; b < 2; ++b) {
       mbar_init(&accf[b], 1);
-      mbar_init(&acce[b], 128);
+      mbar_init(&acce[b], 32 * kRowEpiWarps);
     }
     mbar_init(wbar, 1);
     *abort_flag = 0;
     fence_mbar_init();
   }
-  for (int i = threadIdx.x; i < N; i += kThreads) s_bias[i] = i < p.cout ? p.bias[i] : 0.0f;
+  for (int i = threadIdx.x; i < N; i += kRowThreads) s_bias[i] = i < p.cout ? p.bias[i] : 0.0f;
   if (p.rgba)
-    for (int i = threadIdx.x; i < 4 * N + 4; i += kThreads)  // rows beyond head_n are zero
+    for (int i = threadIdx.x; i < 4 * N + 4; i += kRowThreads)  // rows beyond head_n are zero
       s_head[i] = i < 4 * N ? (i < p.head_n * N ? p.head_w[i] : 0.0f) : (i - 4 * N < p.head_n ? p.head_b[i - 4 * N] : 0.0f);
   if (F8)
-    for (int i = threadIdx.x; i < N; i += kThreads) s_wsc[i] = i < p.cout ? p.w_scale[i] : 0.0f;
+    for (int i = threadIdx.x; i < N; i += kRowThreads) s_wsc[i] = i < p.cout ? p.w_scale[i] : 0.0f;
   const int nbuf = rp.nbuf;
   const uint32_t tmem_cols = (uint32_t)(nbuf * Cfg::kBufCols);
   if (warp == 1) tmem_alloc(tmem_slot, tmem_cols);
@@ -741,7 +745,9 @@ __global__ void __launch_bounds__(kThreads, 2)
       int s = 0, buf = 0;
       uint32_t ph = 0, aph = 0;
       bool ok = mbar_wait(wbar, 0u, abort_flag);
-      const uint32_t wbase = smem_u32(wsm);
+      // operand descriptors advance by constants (rebuilt per MMA they held its issue at ~150 cycles)
+      const uint64_t w_desc = umma_desc<KCB>(smem_u32(wsm)), a_desc = umma_desc<KCB>(smem_u32(stages));
+      const uint32_t w_dx = (uint32_t)(cpt * 3 * N * KCB) >> 4;  // weight blocks of the next horizontal tap
       for (int u = blockIdx.x; ok && u < rp.n_units && !*abort_flag; u += gridDim.x) {
         // the epilogue clears the accumulators (phase 0 = the initial clear)
         if (!mbar_wait(&acce[buf], aph, abort_flag)) break;
@@ -759,14 +765,12 @@ __global__ void __launch_bounds__(kThreads, 2)
               break;
             }
             tc_fence_after();
-            const uint32_t a0 = smem_u32(stages + (size_t)s * kStage);
+            const uint64_t a = a_desc + (uint32_t)(s * (kStage >> 4));
+            uint64_t w = w_desc + (uint32_t)(((c * 3 + lo) * N * KCB) >> 4);
 #pragma unroll
-            for (int dxi = 0; dxi < 3; ++dxi) {
-              const uint32_t bw = wbase + (uint32_t)((wblk(0, dxi, c) + lo) * N * KCB);
+            for (int dxi = 0; dxi < 3; ++dxi, w += w_dx)
 #pragma unroll
-              for (int kk = 0; kk < KCB / 32; ++kk)
-                umma<F8>(dj, umma_desc<KCB>(a0 + dxi * KCB + kk * 32), umma_desc<KCB>(bw + kk * 32), idesc, 1u);
-            }
+              for (int kk = 0; kk < KCB / 32; ++kk) umma<F8>(dj, a + ((dxi * KCB + kk * 32) >> 4), w + kk * 2, idesc, 1u);
             umma_commit(&empty[s]);
             if (++s == S) {
               s = 0;
@@ -786,7 +790,10 @@ __global__ void __launch_bounds__(kThreads, 2)
   } else {
     // ------------------------------------------------------------ epilogue
     grid_dep_wait();  // the output tensors may still be read by the previous layer
-    const int qd = warp & 3;
+    // two warps per TMEM lane quarter, each two of the unit's four rows: a row
+    // takes a warp ~1700 cycles (its loads, transposes and stores one after the
+    // other), four of them longer than the unit's MMAs
+    const int qd = warp & 3, r0 = ((warp - 2) >> 2) * (kRows / 2);
     const int m = qd * 32 + lane;
     const uint32_t tq = tmem_base + ((uint32_t)(qd * 32) << 16);  // this warp's lane quarter
     const float in_s = F8 ? *p.in_scale : 1.0f;
@@ -804,7 +811,7 @@ __global__ void __launch_bounds__(kThreads, 2)
       if (!mbar_wait(&accf[buf], aph, abort_flag, 256)) break;
       tc_fence_after();
       const int y0 = (u / p.tiles_per_row) * kRows, x = (u % p.tiles_per_row) * 128 + m;
-      for (int r = 0; r < kRows; ++r) {
+      for (int r = r0; r < r0 + kRows / 2; ++r) {
         const int slot = kRows - 1 - r;
         const uint32_t ta = tq + (uint32_t)(buf * Cfg::kBufCols + slot * N);
         if (y0 + r < p.H) {
@@ -1073,14 +1080,14 @@ art_status launch_rows(art_ctx* ctx, const TcConv& c) {
   rp.cpt = c.cin / Cfg::KC;
   rp.n_units = ((c.H + kRows - 1) / kRows) * p.tiles_per_row;
   rp.w_bytes = 9 * rp.cpt * N * KCB;
-  const int tail =
-      8 * (2 * 24 + 5) + 16 + 4 * N + 16 + 4 * (4 * 32 + 4) + 4 * N + 16 + (F8 ? 0 : 4 * 32 * 16 * RowOut<N, F8>::U);
+  const int tail = 8 * (2 * 24 + 5) + 16 + 4 * N + 16 + 4 * (4 * 32 + 4) + 4 * N + 16 +
+                   (F8 ? 0 : kRowEpiWarps * 32 * 16 * RowOut<N, F8>::U);
   // two CTAs per SM (two issuing threads, one accumulator buffer each) when
   // the resident weights and three input rows fit in half the shared memory
   const int half = 232448 / 2 - 1024 - rp.w_bytes - tail;
   auto kfn = conv_rows_kernel<N, KCB, F8>;
   cudaFuncAttributes fa;
-  const bool regs2 = cudaFuncGetAttributes(&fa, kfn) == cudaSuccess && 2 * kThreads * fa.numRegs <= 65536;
+  const bool regs2 = cudaFuncGetAttributes(&fa, kfn) == cudaSuccess && 2 * kRowThreads * fa.numRegs <= 65536;
   // (at least three input rows in flight per CTA) and both CTAs' registers fit
   const int ctas = (half >= 3 * Cfg::kStageBytes && regs2) ? 2 : 1;
   const int avail = 232448 / ctas - 1024 - rp.w_bytes - tail;
@@ -1091,7 +1098,7 @@ art_status launch_rows(art_ctx* ctx, const TcConv& c) {
   cudaError_t e = cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return cuda_fail(ctx, e, "conv_rows shared memory attribute");
   const int grid = std::min(rp.n_units, ctas * ctx->num_sms);
-  ART_LAUNCH_PDL(ctx, F8 ? "conv_tc_fp8" : "conv_tc", kfn, grid, kThreads, smem, tmA, tmB, rp);
+  ART_LAUNCH_PDL(ctx, F8 ? "conv_tc_fp8" : "conv_tc", kfn, grid, kRowThreads, smem, tmA, tmB, rp);
   return ART_OK;
 }
 
