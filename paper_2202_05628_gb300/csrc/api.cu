@@ -35,6 +35,16 @@ bool is_device_ptr(const void* p) {
   return at.type == cudaMemoryTypeDevice || at.type == cudaMemoryTypeManaged;
 }
 
+// Host memory that CUDA does not know (neither pinned nor managed).
+static bool pageable(const void* p) {
+  cudaPointerAttributes at;
+  if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return at.type == cudaMemoryTypeUnregistered;
+}
+
 art_status ensure(art_ctx* ctx, void** p, size_t* have, size_t need, const char* what) {
   if (*p && *have >= need) return ART_OK;
   if (*p) cudaFree(*p);
@@ -485,14 +495,21 @@ art_status art_load_skeleton(art_ctx* ctx, int J, const int32_t* parent, const f
   for (int j = 1; j < J; ++j)
     if (par[j] < 0 || par[j] >= j) return fail(ctx, ART_ERR_INVALID_ARG, "parent[%d]=%d must be in [0, %d)", j, par[j], j);
   art_status st;
-  if ((st = alloc(ctx, &ctx->d_skel, (size_t)4 * J, "skeleton")) != ART_OK) return st;
+  if ((st = alloc(ctx, &ctx->d_skel, (size_t)5 * J, "skeleton")) != ART_OK) return st;
   if ((st = alloc(ctx, &ctx->d_pose, (size_t)3 * J + 6, "pose")) != ART_OK) return st;
   if ((st = alloc(ctx, &ctx->d_G, (size_t)12 * J, "joint transforms")) != ART_OK) return st;
-  float host[4 * kMaxJoints];
-  for (int j = 0; j < J; ++j) host[j] = (float)par[j];
+  float host[5 * kMaxJoints];
+  int levels = 0;
+  for (int j = 0; j < J; ++j) {
+    host[j] = (float)par[j];
+    const int l = par[j] < 0 ? 0 : (int)host[4 * J + par[j]] + 1;  // (parents precede children)
+    host[4 * J + j] = (float)l;
+    levels = std::max(levels, l + 1);
+  }
   memcpy(host + J, rest, sizeof(float) * 3 * J);
-  e = cudaMemcpy(ctx->d_skel, host, sizeof(float) * 4 * J, cudaMemcpyHostToDevice);
+  e = cudaMemcpy(ctx->d_skel, host, sizeof(float) * 5 * J, cudaMemcpyHostToDevice);
   if (e != cudaSuccess) return cuda_fail(ctx, e, "upload skeleton");
+  ctx->skel_levels = levels;
   ctx->J = J;
   memcpy(ctx->parent, par, sizeof(int32_t) * J);
   memcpy(ctx->rest, rest, sizeof(float) * 3 * J);
@@ -541,9 +558,22 @@ art_status art_set_pose(art_ctx* ctx, const float* axis_angle, const float R[3],
   if (!axis_angle || !R || !T) return fail(ctx, ART_ERR_INVALID_ARG, "null pose array");
   int J = ctx->J;
   art_status st;
-  if ((st = copy_in(ctx, ctx->d_pose, axis_angle, sizeof(float) * 3 * J, "copy pose")) != ART_OK) return st;
-  if ((st = copy_in(ctx, ctx->d_pose + 3 * J, R, sizeof(float) * 3, "copy pose R")) != ART_OK) return st;
-  if ((st = copy_in(ctx, ctx->d_pose + 3 * J + 3, T, sizeof(float) * 3, "copy pose T")) != ART_OK) return st;
+  // pageable host arrays are read now and travel with the kernel; pinned and
+  // device arrays are read by the stream, as is every pose under capture (a
+  // graph's replay reads the arrays again)
+  PoseArg arg;
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  const bool by_arg = pageable(axis_angle) && pageable(R) && pageable(T) &&
+                      cudaStreamIsCapturing(ctx->stream, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone;
+  if (by_arg) {
+    memcpy(arg.v, axis_angle, sizeof(float) * 3 * J);
+    memcpy(arg.v + 3 * J, R, sizeof(float) * 3);
+    memcpy(arg.v + 3 * J + 3, T, sizeof(float) * 3);
+  } else if ((st = copy_in(ctx, ctx->d_pose, axis_angle, sizeof(float) * 3 * J, "copy pose")) != ART_OK ||
+             (st = copy_in(ctx, ctx->d_pose + 3 * J, R, sizeof(float) * 3, "copy pose R")) != ART_OK ||
+             (st = copy_in(ctx, ctx->d_pose + 3 * J + 3, T, sizeof(float) * 3, "copy pose T")) != ART_OK) {
+    return st;
+  }
   if (!ctx->jidx_ok) {  // joint indices against J: once per octree/skeleton pair
     cudaMemsetAsync(ctx->d_status + 7, 0, sizeof(unsigned long long), ctx->stream);
     check_jidx_kernel<<<(unsigned)((ctx->n + 255) / 256), 256, 0, ctx->stream>>>(ctx->n, ctx->d_jidx, J, ctx->d_status + 7);
@@ -553,7 +583,7 @@ art_status art_set_pose(art_ctx* ctx, const float* axis_angle, const float R[3],
       return fail(ctx, ART_ERR_INVALID_ARG, "%llu voxels reference joints >= J=%d", ctx->h_status[7], J);
     ctx->jidx_ok = true;
   }
-  launch_fk(ctx);  // (zeroes the pose's counters, kStDegenerate and kStRmax)
+  launch_fk(ctx, by_arg ? &arg : nullptr);  // (zeroes the pose's counters, kStDegenerate and kStRmax)
   launch_lbs(ctx);
   if (ctx->cfg.index == ART_INDEX_GRID) {
     if (ctx->grid_slots < 2 * ctx->n) {

@@ -167,7 +167,8 @@ struct art_ctx {
   int J = 0;
   int32_t parent[art::kMaxJoints];
   float rest[art::kMaxJoints * 3];
-  float* d_skel = nullptr;      // parent (as float bits) + rest, uploaded once
+  float* d_skel = nullptr;      // parents (as floats), rest, tree levels; uploaded once
+  int skel_levels = 0;
   float* d_pose = nullptr;      // J*3 + 6
   float* d_G = nullptr;         // [J][12]
 
@@ -301,7 +302,12 @@ void prof_begin(art_ctx* ctx, const char* name);
 void prof_end(art_ctx* ctx);
 
 // ---- kernels: LBS (lbs.cu)
-void launch_fk(art_ctx* ctx);
+// A pose as kernel arguments: r[J][3], R[3], T[3].
+struct PoseArg {
+  float v[3 * kMaxJoints + 6];
+};
+// With arg set, the pose comes with the launch and is also stored in d_pose.
+void launch_fk(art_ctx* ctx, const PoseArg* arg = nullptr);
 void launch_lbs(art_ctx* ctx);
 // The paper's per-frame index after LBS: snap each placed voxel's warped
 // centre to the leaf lattice (hash table of cells, the smallest id wins a

@@ -30,13 +30,17 @@ __device__ void rodrigues(const float* r, float* R) {
 }
 
 // One thread per joint forms its local transform L_j = [R(r_j) | rest_j -
-// rest_parent] (the root's premultiplied by the global [R | T]); one thread
-// then walks the tree (parents precede children), M_j = M_parent L_j, and
-// every joint writes G_j = M_j [I | -rest_j].
-// skel: J parent indices stored as floats, then rest[J][3]; pose: r[J][3], R[3], T[3].
-__global__ void __launch_bounds__(kMaxJoints) fk_kernel(int J, const float* __restrict__ skel,
-                                                        const float* __restrict__ pose, float* __restrict__ G,
-                                                        unsigned long long* __restrict__ status) {
+// rest_parent] (the root's premultiplied by the global [R | T]); the tree is
+// then composed level by level, M_j = M_parent L_j, and every joint writes
+// G_j = M_j [I | -rest_j].
+// skel: J parent indices stored as floats, rest[J][3], J tree levels; pose:
+// r[J][3], R[3], T[3], read from `pose`, or (ARG) from the launch's arguments
+// and stored there for later readers: a pose in pageable host memory needs no
+// copies before the kernel (three of them cost a small frame ~5 us).
+template <bool ARG>
+__global__ void __launch_bounds__(kMaxJoints) fk_kernel(int J, int levels, const float* __restrict__ skel,
+                                                        const __grid_constant__ PoseArg arg, float* __restrict__ pose,
+                                                        float* __restrict__ G, unsigned long long* __restrict__ status) {
   ART_PDL_ENTRY();
   if (threadIdx.x == 0) {  // the pose's counters, accumulated by the skinning that follows
     status[kStDegenerate] = 0ull;
@@ -44,22 +48,24 @@ __global__ void __launch_bounds__(kMaxJoints) fk_kernel(int J, const float* __re
   }
   __shared__ float sL[kMaxJoints][12];
   __shared__ float sM[kMaxJoints][12];
-  __shared__ int sp[kMaxJoints];
   __shared__ float srest[kMaxJoints][3];
   const int j = threadIdx.x;
   const bool on = j < J;
-  int p = -1;
+  if constexpr (ARG)
+    for (int k = j; k < 3 * J + 6; k += kMaxJoints) pose[k] = arg.v[k];
+  auto pose_at = [&](int k) { return ARG ? arg.v[k] : pose[k]; };
+  int p = -1, level = -1;
   float r[3] = {0.f, 0.f, 0.f}, rg[3], Tg[3];
   if (on) {
     p = (int)skel[j];
-    sp[j] = p;
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
       srest[j][a] = skel[J + 3 * j + a];
-      r[a] = pose[3 * j + a];
-      rg[a] = pose[3 * J + a];
-      Tg[a] = pose[3 * J + 3 + a];
+      r[a] = pose_at(3 * j + a);
+      rg[a] = pose_at(3 * J + a);
+      Tg[a] = pose_at(3 * J + 3 + a);
     }
+    level = (int)skel[4 * J + j];
   }
   __syncthreads();
   if (on) {
@@ -83,14 +89,13 @@ __global__ void __launch_bounds__(kMaxJoints) fk_kernel(int J, const float* __re
     }
   }
   __syncthreads();
-  if (j == 0) {
-    for (int k = 0; k < J; ++k) {
-      const int q = sp[k];
+  for (int l = 0; l < levels; ++l) {
+    if (level == l) {
       float P[12];
 #pragma unroll
-      for (int m = 0; m < 12; ++m) P[m] = sM[q >= 0 ? q : k][m];
-      const float* L = sL[k];
-      float* Mk = sM[k];
+      for (int m = 0; m < 12; ++m) P[m] = sM[p >= 0 ? p : j][m];
+      const float* L = sL[j];
+      float* Mk = sM[j];
 #pragma unroll
       for (int a = 0; a < 3; ++a) {
 #pragma unroll
@@ -99,8 +104,8 @@ __global__ void __launch_bounds__(kMaxJoints) fk_kernel(int J, const float* __re
         Mk[a * 4 + 3] = P[a * 4 + 0] * L[3] + P[a * 4 + 1] * L[7] + P[a * 4 + 2] * L[11] + P[a * 4 + 3];
       }
     }
+    __syncthreads();
   }
-  __syncthreads();
   if (on) {
     const float* M = sM[j];
 #pragma unroll
@@ -474,8 +479,13 @@ void launch_grid_snap(art_ctx* ctx) {
              ctx->origin[1], ctx->origin[2], ctx->h, ctx->d_gkeys, ctx->d_gvals, mask, ctx->d_status);
 }
 
-void launch_fk(art_ctx* ctx) {
-  ART_LAUNCH_PDL(ctx, "fk", fk_kernel, 1, kMaxJoints, 0, ctx->J, ctx->d_skel, ctx->d_pose, ctx->d_G, ctx->d_status);
+void launch_fk(art_ctx* ctx, const PoseArg* arg) {
+  if (arg)
+    ART_LAUNCH_PDL(ctx, "fk", fk_kernel<true>, 1, kMaxJoints, 0, ctx->J, ctx->skel_levels, ctx->d_skel, *arg, ctx->d_pose,
+                   ctx->d_G, ctx->d_status);
+  else
+    ART_LAUNCH_PDL(ctx, "fk", fk_kernel<false>, 1, kMaxJoints, 0, ctx->J, ctx->skel_levels, ctx->d_skel, PoseArg{},
+                   ctx->d_pose, ctx->d_G, ctx->d_status);
 }
 
 void launch_lbs(art_ctx* ctx) {
