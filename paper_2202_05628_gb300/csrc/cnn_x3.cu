@@ -34,11 +34,11 @@
 // registers, its drains outlast the other row's MMAs, and small images have
 // half as many units.
 //
-// Bounds: shared-memory bandwidth (operand reads are ~90 % of it at these N,
-// the TMA boxes come on top) at 50-56 % tensor-pipe time for N = 64; for
-// N = 32 the drain and epilogue latencies between its short blocks (32 %).
-// Measured: FP32 frame of 1M voxels at 1024x1024 10.22 ms with the CUDA-core
-// kernels (36 TFLOP/s) -> 1.96 ms; the U-Net at 424x248 1716 -> 398 us.
+// Bounds: shared-memory bandwidth (operand reads are ~125 B a clock at these N,
+// the TMA boxes and the staged stores come on top): 49-61 % tensor-pipe time for
+// N = 64; for N = 32 (36-42 %) also the epilogue between its short units.
+// Measured: FP32 frame of 1M voxels at 1024x1024 10.21 ms with the CUDA-core
+// kernels (36 TFLOP/s) -> 1.74 ms; the U-Net at 424x248 1720 -> 351 us.
 //
 // A result that is not finite (an infinite or NaN input, or parts whose
 // products overflow) is recomputed as the FP32 FMA chain over taps and
@@ -466,115 +466,116 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
   } else if (warp == 1) {
     // ---------------------------------------------------------------- MMA
-    if (lane == 0) {
-      RingPos ra, rb;
-      uint32_t aph = 0;  // both rows' accumulators are used once per K block
-      bool ok = true;
-      const uint64_t a_base = umma_desc<kKCB>(smem_u32(sA)), b_base = umma_desc<kKCB>(smem_u32(sB));
-      auto wait_a = [&](const RingPos& r) { ok = ok && mbar_wait(&fullA[r.i], r.ph, abort_flag); };
-      auto wait_b = [&](const RingPos& r) { ok = ok && mbar_wait(&fullB[r.i], r.ph, abort_flag); };
-      auto wait_acc = [&](int r) { ok = ok && mbar_wait(&acce[r], aph ^ 1u, abort_flag); };
-      auto A = [&](const RingPos& r, int off) { return a_base + (uint32_t)((r.i * kSlotA + off * kKCB) >> 4); };
-      auto B = [&](const RingPos& r) { return b_base + (uint32_t)((r.i * C::kSlotB) >> 4); };
-      const uint32_t d[2] = {tmem_base, tmem_base + (uint32_t)C::kSet};
-      for (int u = blockIdx.x; ok && u < p.n_units && !*abort_flag; u += gridDim.x) {
-        Start start = kFreshAll;  // of a block's first tap
-        if constexpr (!SUB) {
-          for (int c = 0; ok && c < p.c0; ++c) {
-            wait_a(ra);
-            for (int dy = 0; ok && dy < 3; ++dy) {
-              RingPos b = rb;
-              wait_acc(0);
-              tc_fence_after();
+    // The whole warp runs the loop and one elected lane issues, so that operand
+    // addresses stay in uniform registers (a lone lane's ~68 cycles per MMA were
+    // more than N = 32 executes in).  The tensor pipe queues about one MMA beyond
+    // the running one, so everything the next row waits for is waited for before
+    // this row's last tap: ~270 cycles between rows were idle.
+    const bool el = elect_one();
+    RingPos ra, rb;
+    uint32_t aph = 0;  // both rows' accumulators are used once per K block
+    bool ok = true;
+    const uint64_t a_base = umma_desc<kKCB>(smem_u32(sA)), b_base = umma_desc<kKCB>(smem_u32(sB));
+    auto wait = [&](uint64_t* bar, uint32_t ph) { ok = ok && __all_sync(0xffffffffu, mbar_wait(bar, ph, abort_flag)); };
+    auto wait_a = [&](const RingPos& r) { wait(&fullA[r.i], r.ph); };
+    auto wait_b = [&](const RingPos& r) { wait(&fullB[r.i], r.ph); };
+    auto A = [&](const RingPos& r, int off) { return a_base + (uint32_t)((r.i * kSlotA + off * kKCB) >> 4); };
+    auto B = [&](const RingPos& r) { return b_base + (uint32_t)((r.i * C::kSlotB) >> 4); };
+    const uint32_t d[2] = {tmem_base, tmem_base + (uint32_t)C::kSet};
+    auto tap = [&](int r, uint64_t a1, uint64_t w1, Start st) {
+      tc_fence_after();
+      if (ok && el) tap_mma<N>(d[r], a1, w1, st);
+    };
+    auto commit = [&](uint64_t* bar) {
+      if (ok && el) umma_commit(bar);
+    };
+    auto free_b = [&]() {  // the weights in hand have served both rows
+      commit(&emptyB[rb.i]);
+      rb.next(C::kSlotsB);
+    };
+    // (the first row's accumulators of a block are waited for in the block before)
+    for (int u = blockIdx.x; ok && u < p.n_units && !*abort_flag; u += gridDim.x) {
+      Start start = kFreshAll;  // of a block's first tap
+      if constexpr (!SUB) {
+        for (int c = 0; ok && c < p.c0; ++c) {
+          wait_a(ra);
+          for (int dy = 0; ok && dy < 3; ++dy) {  // first row: input row dy of the four; second: dy + 1
+            RingPos b = rb, an = ra;
+            an.next(C::kSlotsA);
 #pragma unroll
-              for (int dx = 0; dx < 3; ++dx) {  // first row: input row dy of the four
-                wait_b(b);
-                tc_fence_after();
-                if (ok) tap_mma<N>(d[0], A(ra, dx), B(b), dx == 0 ? start : kGoOn);
-                b.next(C::kSlotsB);
-              }
-              if (!ok) break;
-              umma_commit(&accf[0]);
-              umma_commit(&emptyA[ra.i]);
-              ra.next(C::kSlotsA);
-              wait_a(ra);
-              wait_acc(1);
-              if (!ok) break;
-              tc_fence_after();
-#pragma unroll
-              for (int dx = 0; dx < 3; ++dx) {  // second row: input row dy + 1
-                tap_mma<N>(d[1], A(ra, dx), B(rb), dx == 0 ? start : kGoOn);
-                umma_commit(&emptyB[rb.i]);
-                rb.next(C::kSlotsB);
-              }
-              umma_commit(&accf[1]);
-              aph ^= 1u;
-              start = kFreshA;
-            }
-            if (!ok) break;
-            umma_commit(&emptyA[ra.i]);
-            ra.next(C::kSlotsA);
-          }
-        } else {
-          for (int k = 0; ok && k < 3 * p.c0; ++k) {  // skip taps: even box E, odd box O
-            const RingPos e = ra;
-            ra.next(C::kSlotsA);
-            const RingPos o = ra;
-            ra.next(C::kSlotsA);
-            RingPos b = rb;
-            wait_a(e);
-            wait_a(o);
-            wait_acc(0);
-            tc_fence_after();
-#pragma unroll
-            for (int dx = 0; dx < 3; ++dx) {  // even column 2j: input columns 2j - 1, 2j, 2j + 1
+            for (int dx = 0; dx < 3; ++dx) {
               wait_b(b);
-              tc_fence_after();
-              if (ok) tap_mma<N>(d[0], dx == 1 ? A(e, 1) : A(o, dx / 2), B(b), dx == 0 ? start : kGoOn);
+              if (dx == 2) {
+                wait_a(an);
+                wait(&acce[1], aph ^ 1u);
+              }
+              tap(0, A(ra, dx), B(b), dx == 0 ? start : kGoOn);
               b.next(C::kSlotsB);
             }
-            if (!ok) break;
-            umma_commit(&accf[0]);
-            wait_acc(1);
-            if (!ok) break;
-            tc_fence_after();
+            commit(&accf[0]);
 #pragma unroll
-            for (int dx = 0; dx < 3; ++dx) {  // odd column 2j + 1: input columns 2j, 2j + 1, 2j + 2
-              tap_mma<N>(d[1], dx == 1 ? A(o, 1) : A(e, 1 + dx / 2), B(rb), dx == 0 ? start : kGoOn);
-              umma_commit(&emptyB[rb.i]);
-              rb.next(C::kSlotsB);
+            for (int dx = 0; dx < 3; ++dx) {
+              if (dx == 2) wait(&acce[0], aph);
+              tap(1, A(an, dx), B(rb), dx == 0 ? start : kGoOn);
+              if (dx == 0) commit(&emptyA[ra.i]);
+              free_b();
             }
-            umma_commit(&accf[1]);
-            umma_commit(&emptyA[e.i]);
-            umma_commit(&emptyA[o.i]);
+            commit(&accf[1]);
             aph ^= 1u;
             start = kFreshA;
+            ra = an;
           }
-          for (int k = 0; ok && k < 2 * p.c1; ++k) {  // low-resolution taps: columns j - 1, j | j, j + 1
-            wait_a(ra);
-            for (int px = 0; ok && px < 2; ++px) {
-              wait_acc(px);
-              tc_fence_after();
+          commit(&emptyA[ra.i]);
+          ra.next(C::kSlotsA);
+        }
+      } else {
+        for (int k = 0; ok && k < 3 * p.c0; ++k) {  // skip taps: even box E, odd box O
+          const RingPos e = ra;
+          ra.next(C::kSlotsA);
+          const RingPos o = ra;
+          ra.next(C::kSlotsA);
+          RingPos b = rb;
+          wait_a(e);
+          wait_a(o);
 #pragma unroll
-              for (int ox = 0; ox < 2; ++ox) {
-                wait_b(rb);
-                if (!ok) break;
-                tc_fence_after();
-                tap_mma<N>(d[px], A(ra, px + ox), B(rb), ox == 0 ? kFreshA : kGoOn);
-                umma_commit(&emptyB[rb.i]);
-                rb.next(C::kSlotsB);
-              }
-              if (ok) umma_commit(&accf[px]);
-            }
-            if (!ok) break;
-            umma_commit(&emptyA[ra.i]);
-            ra.next(C::kSlotsA);
-            aph ^= 1u;
+          for (int dx = 0; dx < 3; ++dx) {  // even column 2j: input columns 2j - 1, 2j, 2j + 1
+            wait_b(b);
+            if (dx == 2) wait(&acce[1], aph ^ 1u);
+            tap(0, dx == 1 ? A(e, 1) : A(o, dx / 2), B(b), dx == 0 ? start : kGoOn);
+            b.next(C::kSlotsB);
           }
+          commit(&accf[0]);
+#pragma unroll
+          for (int dx = 0; dx < 3; ++dx) {  // odd column 2j + 1: input columns 2j, 2j + 1, 2j + 2
+            if (dx == 2) wait(&acce[0], aph);
+            tap(1, dx == 1 ? A(o, 1) : A(e, 1 + dx / 2), B(rb), dx == 0 ? start : kGoOn);
+            free_b();
+          }
+          commit(&accf[1]);
+          commit(&emptyA[e.i]);
+          commit(&emptyA[o.i]);
+          aph ^= 1u;
+          start = kFreshA;
+        }
+        for (int k = 0; ok && k < 2 * p.c1; ++k) {  // low-resolution taps: columns j - 1, j | j, j + 1
+          wait_a(ra);
+#pragma unroll
+          for (int px = 0; px < 2; ++px) {
+#pragma unroll
+            for (int ox = 0; ox < 2; ++ox) {
+              wait_b(rb);
+              if (ox == 1) wait(&acce[px ^ 1], px == 0 ? aph ^ 1u : aph);
+              tap(px, A(ra, px + ox), B(rb), ox == 0 ? kFreshA : kGoOn);
+              free_b();
+            }
+            commit(&accf[px]);
+          }
+          commit(&emptyA[ra.i]);
+          ra.next(C::kSlotsA);
+          aph ^= 1u;
         }
       }
     }
-    __syncwarp();
   } else {
     // ---------------------------------------------------------------- epilogue
     const int g = (warp - 2) >> 2;     // this group's row (sub: column phase)
