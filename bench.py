@@ -242,8 +242,8 @@ def roofline(kt, stats, peaks, form, n_vox, C, frames, conv_launch_ms=None):
         out.update(avg_ms=avg_ms, avg_ms_from="shading network called back to back, time / its 14 "
                    "convolution launches (its one pooling launch included)")
     if name.startswith("conv"):
-        # the FLOPs the network executes (BF16: the sub-pixel decoder convolution at level 0)
-        flops = unet_flops(RES, RES, subpixel=(net == "bf16"))
+        # the FLOPs the network executes (BF16 and FP32: the decoders' first convolutions in sub-pixel form)
+        flops = unet_flops(RES, RES, subpixel=(net in ("bf16", "f32")))
         per_launch = flops * frames / max(nl, 1)
         out.update(flops_per_frame=flops, flops_plain_definition=unet_flops(RES, RES))
         ach = per_launch / (avg_ms * 1e-3) / 1e12
@@ -256,7 +256,7 @@ def roofline(kt, stats, peaks, form, n_vox, C, frames, conv_launch_ms=None):
         bf16 = peaks.get(key, 1900.0 if isolated else 1700.0)
         kind = "burst" if isolated else "sustained"
         if net == "f32":
-            peak, bound, note = 2.0 * 152 * 128 * 2.07e9 / 1e12, "alu", "FP32 FMA issue rate of the CUDA cores"
+            peak, bound, note = bf16 / 6.0, "tensor", f"{src} {kind} BF16 / 6 (six part products per FP32 product)"
         elif net == "fp8":
             peak, bound, note = 2.0 * bf16, "tensor", f"{src} {kind} BF16 x 2 (nominal FP8 / BF16 ratio)"
         else:

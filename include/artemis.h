@@ -241,7 +241,8 @@ typedef struct {
  *       with art_shade_with_opacity (it needs A); F32 or BF16 only.
  * params: float array, for every layer in execution order its weights
  *   [Cout][k][k][Cin] followed by its bias [Cout]; n_params must match.
- * compute_dtype: ART_F32 (CUDA-core FP32), ART_BF16 (tensor cores, BF16
+ * compute_dtype: ART_F32 (FP32: on the tensor cores as exact three-part BF16
+ *   products where the widths allow, else on CUDA cores), ART_BF16 (tensor cores, BF16
  *   operands, FP32 accumulation) or ART_FP8 (U-Net only: E4M3 operands,
  *   FP32 accumulation, per-output-channel weight scales max|w_co| / 448 and
  *   per-tensor activation scales; each art_shade quantises with the scales
