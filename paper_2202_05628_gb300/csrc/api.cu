@@ -811,6 +811,21 @@ art_status art_render_views(art_ctx* ctx, int nv, const int* views, void* const*
                         k == 0);
   }
   launch_bin_views(ctx, vs, total);
+  {  // the clear of the views' empty tiles on the side stream beside the bucket sort (as sort_beside)
+    if ((st = ensure_side(ctx)) != ART_OK) return st;
+    cudaStream_t main_stream = ctx->stream;
+    cudaEventRecord(ctx->ev_fork, main_stream);
+    cudaStreamWaitEvent(ctx->side, ctx->ev_fork, 0);
+    ctx->stream = ctx->side;
+    for (int k = 0; k < nv && st == ART_OK; ++k)
+      st = launch_composite_clear(ctx, vs.v[k], vs.F[k], F_dtype, vs.A[k], ctx->d_ranges + vs.toff[k]);
+    cudaEventRecord(ctx->ev_join, ctx->side);
+    ctx->stream = main_stream;
+    launch_tile_sort_views(ctx, vs, total);
+    cudaStreamWaitEvent(main_stream, ctx->ev_join, 0);
+    ctx->pose_bias_side = false;  // (the join follows the side stream's pose bias too)
+    if (st != ART_OK) return st;
+  }
   if ((st = launch_composite_views(ctx, vs, F_dtype)) != ART_OK) return st;
   return launch_check(ctx, "render_views");
 }

@@ -600,7 +600,7 @@ __device__ __forceinline__ unsigned long long bucket_entry(uint32_t key, uint32_
 // (quantum, voxel id) pairs in its bin; larger bins are sorted by one warp.
 __device__ void block_sort_bucket(uint32_t* __restrict__ keys, uint32_t* __restrict__ vals, uint32_t n,
                                   uint32_t qmask, uint32_t thi, unsigned long long* S) {
-  __shared__ uint32_t s_start[kSortBins], s_cur[kSortBins];
+  __shared__ __align__(16) uint32_t s_start[kSortBins], s_cur[kSortBins];
   __shared__ uint32_t s_lo[kTileSortWarps], s_hi[kTileSortWarps];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const bool regs = n <= (uint32_t)kSortRegs;
@@ -632,7 +632,8 @@ __device__ void block_sort_bucket(uint32_t* __restrict__ keys, uint32_t* __restr
     s_lo[warp] = lo;
     s_hi[warp] = hi;
   }
-  for (int b = threadIdx.x; b < kSortBins; b += kTileSortThreads) s_cur[b] = 0;
+  for (int b = threadIdx.x; b < kSortBins / 4; b += kTileSortThreads)
+    reinterpret_cast<uint4*>(s_cur)[b] = make_uint4(0u, 0u, 0u, 0u);
   __syncthreads();
   lo = s_lo[0];
   hi = s_hi[0];
@@ -654,20 +655,21 @@ __device__ void block_sort_bucket(uint32_t* __restrict__ keys, uint32_t* __restr
   }
   __syncthreads();
   {  // exclusive scan of the bin counts
-    constexpr int kPer = kSortBins / kTileSortThreads;
-    uint32_t c[kPer], t = 0;
-    const int b0 = threadIdx.x * kPer;
+    constexpr int kPer = kSortBins / kTileSortThreads / 4;  // 16-byte rows of four bins per thread
+    uint4 c[kPer];
+    uint32_t t = 0;
 #pragma unroll
     for (int e = 0; e < kPer; ++e) {
-      c[e] = s_cur[b0 + e];
-      t += c[e];
+      c[e] = reinterpret_cast<const uint4*>(s_cur)[threadIdx.x * kPer + e];
+      t += (c[e].x + c[e].y) + (c[e].z + c[e].w);
     }
     uint32_t run = block_exclusive_scan(t, nullptr);
 #pragma unroll
     for (int e = 0; e < kPer; ++e) {
-      s_start[b0 + e] = run;
-      s_cur[b0 + e] = run;
-      run += c[e];
+      const uint4 r = make_uint4(run, run + c[e].x, run + c[e].x + c[e].y, run + c[e].x + c[e].y + c[e].z);
+      reinterpret_cast<uint4*>(s_start)[threadIdx.x * kPer + e] = r;
+      reinterpret_cast<uint4*>(s_cur)[threadIdx.x * kPer + e] = r;
+      run = r.w + c[e].w;
     }
   }
   __syncthreads();
@@ -814,8 +816,11 @@ void launch_bin_views(art_ctx* ctx, const ViewSet& vs, int64_t ntiles) {
                ctx->d_q_v + o, vs.v[k], ctx->inst_cap, vs.toff[k], ctx->d_toff, ctx->d_keys, ctx->d_vals,
                ctx->d_status, (const uint32_t*)nullptr, (const float*)nullptr, (float*)nullptr);
   }
+}
+
+void launch_tile_sort_views(art_ctx* ctx, const ViewSet& vs, int64_t ntiles) {
   ART_LAUNCH_PDL(ctx, "tile_sort", tile_sort_kernel, 2 * ctx->num_sms, kTileSortThreads, kTileSortSmem * 8, ctx->d_ranges,
-             ctx->d_sortlist, nt, vs.v[0].depth_bits, ctx->d_keys, ctx->d_vals, ctx->d_sort_tmp, ctx->d_status);
+             ctx->d_sortlist, (int)ntiles, vs.v[0].depth_bits, ctx->d_keys, ctx->d_vals, ctx->d_sort_tmp, ctx->d_status);
 }
 
 int launch_sort(art_ctx* ctx, uint32_t* k0, uint32_t* v0, uint32_t* k1, uint32_t* v1, int64_t n, int key_bits,

@@ -978,9 +978,8 @@ uint32_t next_xstamp(art_ctx* ctx, size_t ntiles) {
   return ctx->xstamp;
 }
 
-// The plain split walk of a batch of views: plan all segments, clear each
-// view's empty tiles, walk all segments with persistent warps, merge the
-// split tiles, then walk the tiles whose stop fell inside a later segment.
+// The plain split walk of a batch of views: plan all segments, walk all
+// segments with persistent warps, merge the split tiles, then walk the tiles whose stop fell inside a later segment.
 template <int C, typename TF, typename TO>
 void views_walk(art_ctx* ctx, const ViewSet& vs) {
   const int ntiles = (int)vs.toff[vs.nv];
@@ -989,12 +988,6 @@ void views_walk(art_ctx* ctx, const ViewSet& vs) {
   zero_words(ctx, kPassWords | bit(kStFallback) | bit(kStExactQ));
   ART_LAUNCH_PDL(ctx, "composite_plan", seg_plan_kernel, (ntiles + 255) / 256, 256, 0, ntiles, ctx->d_ranges, ctx->seg_len,
              0, ctx->d_seg, ctx->d_items, ctx->d_multi, ctx->d_status);
-  for (int k = 0; k < vs.nv; ++k) {
-    const ViewParams& v = vs.v[k];
-    auto cfn = composite_clear_kernel<C, TO>;
-    ART_LAUNCH_PDL(ctx, "composite_clear", cfn, (v.tiles_x * v.tiles_y + 7) / 8, 256, 0, ctx->d_ranges + vs.toff[k], v,
-               (TO*)vs.F[k], vs.A[k]);
-  }
   auto kfn = composite_split_views_kernel<C, TF, TO>;
   ART_LAUNCH_PDL(ctx, "composite", kfn, ctx->composite_blocks, 32, 0, ctx->d_vset, ctx->d_ranges, ctx->d_seg, ctx->d_items,
              ctx->d_keys, ctx->d_vals, ctx->d_rec, ctx->d_rect_v, feat, ctx->cfg.tau, ctx->d_status, ctx->d_part,
@@ -1266,25 +1259,27 @@ int composite_blocks_per_sm(int C, int feat_bytes) {
 
 namespace {
 template <int C>
-void clear_c(art_ctx* ctx, const ViewParams& v, void* F, int F_dtype, float* A) {
+void clear_c(art_ctx* ctx, const ViewParams& v, void* F, int F_dtype, float* A, const uint2* ranges) {
   const int ntiles = v.tiles_x * v.tiles_y;
   if (F_dtype == ART_F32) {
-    ART_LAUNCH_PDL(ctx, "composite_clear", (composite_clear_kernel<C, float>), (ntiles + 7) / 8, 256, 0, ctx->d_ranges,
-                   v, (float*)F, A);
+    ART_LAUNCH_PDL(ctx, "composite_clear", (composite_clear_kernel<C, float>), (ntiles + 7) / 8, 256, 0, ranges, v,
+                   (float*)F, A);
   } else {
     ART_LAUNCH_PDL(ctx, "composite_clear", (composite_clear_kernel<C, __nv_bfloat16>), (ntiles + 7) / 8, 256, 0,
-                   ctx->d_ranges, v, (__nv_bfloat16*)F, A);
+                   ranges, v, (__nv_bfloat16*)F, A);
   }
 }
 }  // namespace
 
-art_status launch_composite_clear(art_ctx* ctx, const ViewParams& v, void* F, int F_dtype, float* A) {
+art_status launch_composite_clear(art_ctx* ctx, const ViewParams& v, void* F, int F_dtype, float* A,
+                                  const uint2* ranges) {
+  if (!ranges) ranges = ctx->d_ranges;
   if (v.tile_w != TSX || v.tile_h != TSY) return fail(ctx, ART_ERR_UNSUPPORTED, "composite: tiles must be 8x4");
   switch (ctx->C) {
-    case 4: clear_c<4>(ctx, v, F, F_dtype, A); break;
-    case 8: clear_c<8>(ctx, v, F, F_dtype, A); break;
-    case 16: clear_c<16>(ctx, v, F, F_dtype, A); break;
-    case 32: clear_c<32>(ctx, v, F, F_dtype, A); break;
+    case 4: clear_c<4>(ctx, v, F, F_dtype, A, ranges); break;
+    case 8: clear_c<8>(ctx, v, F, F_dtype, A, ranges); break;
+    case 16: clear_c<16>(ctx, v, F, F_dtype, A, ranges); break;
+    case 32: clear_c<32>(ctx, v, F, F_dtype, A, ranges); break;
     default: return fail(ctx, ART_ERR_UNSUPPORTED, "composite: C=%d not built (4, 8, 16, 32)", ctx->C);
   }
   return ART_OK;

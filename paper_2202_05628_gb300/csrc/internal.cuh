@@ -342,8 +342,10 @@ void launch_bin(art_ctx* ctx, const ViewParams& v, const uint32_t* hbin = nullpt
 void launch_tile_sort(art_ctx* ctx, const ViewParams& v);
 // Binning of a batch of views in one tile space (ntiles in all, joint
 // depth_bits): one scan of all tiles' counts, one scatter per view (its
-// instances keyed by global tile), one sort of all buckets.
+// instances keyed by global tile); the sort of all buckets is a call of its
+// own, so that work which needs only the ranges can run beside it.
 void launch_bin_views(art_ctx* ctx, const ViewSet& vs, int64_t ntiles);
+void launch_tile_sort_views(art_ctx* ctx, const ViewSet& vs, int64_t ntiles);
 // Radix sort of n pairs ping-ponging between (k0, v0) and (k1, v1); returns
 // the index (0 or 1) of the buffer holding the result.  counts and look: scratch
 // of sort_count_words() and sort_look_words(n) words.
@@ -370,11 +372,14 @@ art_status launch_composite_skip(art_ctx* ctx, const ViewParams& v, void* F, int
 // Zero F and A of the tiles without instances (needs only the tile ranges);
 // a composite that follows on the same frame with ctx->f_cleared set skips
 // its own clear.
-art_status launch_composite_clear(art_ctx* ctx, const ViewParams& v, void* F, int F_dtype, float* A);
+// ranges: the view's tile ranges (null: d_ranges).
+art_status launch_composite_clear(art_ctx* ctx, const ViewParams& v, void* F, int F_dtype, float* A,
+                                  const uint2* ranges = nullptr);
 // Labels of the plain composite (labels [H][W][3], bins [H][W][2]; either may be null).
 art_status launch_composite_labels(art_ctx* ctx, const ViewParams& v, float* labels, uint8_t* bins);
 // Plain composite of a batch of views in one split pass over the joint tile
-// space (after launch_bin_views); vs is the host copy of *ctx->d_vset.
+// space (after launch_bin_views, launch_tile_sort_views and the clear of every
+// view's empty tiles); vs is the host copy of *ctx->d_vset.
 art_status launch_composite_views(art_ctx* ctx, const ViewSet& vs, int F_dtype);
 // One-warp blocks of the composite walk that fit on an SM (C channels of feat_bytes).
 int composite_blocks_per_sm(int C, int feat_bytes);
