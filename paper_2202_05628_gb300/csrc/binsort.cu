@@ -53,7 +53,9 @@ __device__ uint32_t block_exclusive_scan(uint32_t v, uint32_t* total) {
 // nearest published prefix is far at first and a walk one tile at a time would
 // take as many memory latencies as there are tiles.  The pairs are brought into
 // digit order in shared memory meanwhile, so that runs of a digit are stored
-// contiguously.
+// contiguously.  900,001 pairs by 32 bits: 168 us with five launches a pass
+// (count, three scans, scatter), 77 now, ~14 a pass: latencies of the ranking,
+// the look-back and the scatter on 220 tiles.
 constexpr int kSortThreads = 256;
 constexpr int kSortWarps = kSortThreads / 32;
 constexpr int kSortRounds = 16;

@@ -32,6 +32,11 @@
 // by side in shared memory.  Zero padding comes from the boxes' out of range
 // pixels (TMA fills zeros), which is exact: an upsampled pixel outside the
 // image maps to a low-resolution one outside it.
+//
+// Bound by shared memory (an MMA of 32 or 64 columns reads its operands at 128
+// bytes a cycle; ~74 cycles per MMA against 43) at 27 % tensor-pipe time.
+// 1024x1024, 96 -> 32 channels: 77 us, 57 without divisions on the issuing
+// threads, 55 with the skip blocks kept once (six stages instead of four).
 #include <cuda.h>
 #include <cudaTypedefs.h>
 
