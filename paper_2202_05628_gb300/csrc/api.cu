@@ -1235,7 +1235,7 @@ art_status art_sync_status(art_ctx* ctx, art_stats* out) {
     return r;
   }
   if (h[kStScanError]) {
-    art_status r = fail(ctx, ART_ERR_CUDA, "binning or sort: %llu look-backs timed out waiting for a predecessor",
+    art_status r = fail(ctx, ART_ERR_CUDA, "binning: %llu tile-scan blocks timed out waiting for a predecessor",
                         h[kStScanError]);
     cudaMemsetAsync(ctx->d_status + kStScanError, 0, sizeof(unsigned long long), ctx->stream);
     cudaStreamSynchronize(ctx->stream);

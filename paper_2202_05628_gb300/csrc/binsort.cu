@@ -51,7 +51,9 @@ __device__ uint32_t block_exclusive_scan(uint32_t v, uint32_t* total) {
 // counts, and thread d looks back over the earlier tiles' counts of digit d,
 // sixteen of them per round: all of a small sort's tiles run at once, so the
 // nearest published prefix is far at first and a walk one tile at a time would
-// take as many memory latencies as there are tiles.  The pairs are brought into
+// take as many memory latencies as there are tiles.  A thread that has waited
+// too long counts the missing tile's keys itself (they stay unchanged during
+// the pass), so that no wait can end in a wrong order.  The pairs are brought into
 // digit order in shared memory meanwhile, so that runs of a digit are stored
 // contiguously.  900,001 pairs by 32 bits: 168 us with five launches a pass
 // (count, three scans, scatter), 77 now, ~14 a pass: latencies of the ranking,
@@ -65,7 +67,10 @@ constexpr int kRadix = 1 << kRadixBits;
 constexpr int kMaxPasses = 4;
 constexpr int kLookBack = 16;            // predecessors read per look-back round
 constexpr int kCountReplicas = 4;        // digit counters per block of the count (lanes of a warp often share a digit)
-constexpr long long kSortSpin = 1 << 22;  // look-back polls before a block gives up
+#ifndef ART_SORT_SPIN  // (a build that sets it to -1 waits for no tile: every count not yet there is made from the keys)
+#define ART_SORT_SPIN (1 << 22)
+#endif
+constexpr long long kSortSpin = ART_SORT_SPIN;  // look-back polls of a thread before it counts missing tiles itself
 
 // What a tile has published of a digit in a pass: nothing, its own count, or
 // the count of all tiles up to it.  The tag names the pass, so one array
@@ -114,13 +119,19 @@ __global__ void __launch_bounds__(kSortThreads) radix_count_kernel(const uint32_
   }
 }
 
+// How many keys of a tile before the last (which alone is not full) have the digit.
+__device__ __noinline__ uint32_t count_tile(const uint32_t* kin, int64_t tile, int shift, uint32_t digit) {
+  uint32_t c = 0;
+  for (int i = 0; i < kSortTile; ++i) c += ((kin[tile * kSortTile + i] >> shift) & (kRadix - 1)) == digit;
+  return c;
+}
+
 template <typename S>
 __global__ void __launch_bounds__(kSortThreads) radix_pass_kernel(const uint32_t* __restrict__ kin,
                                                                   const uint32_t* __restrict__ vin,
                                                                   uint32_t* __restrict__ kout,
                                                                   uint32_t* __restrict__ vout, int64_t n, int pass,
-                                                                  uint32_t* __restrict__ counts, S* look,
-                                                                  unsigned long long* __restrict__ err) {
+                                                                  uint32_t* __restrict__ counts, S* look) {
   ART_PDL_ENTRY();
   constexpr int kShift = LookWord<S>::kShift;
   __shared__ uint32_t wh[kSortWarps][kRadix];  // per warp: digit counts, then offsets within the tile's digit
@@ -216,10 +227,7 @@ __global__ void __launch_bounds__(kSortThreads) radix_pass_kernel(const uint32_t
     }
     if (end) break;
     q -= used;
-    if (used == 0 && ++spin > kSortSpin) {
-      if (err) atomicAdd(err, 1ull);
-      break;
-    }
+    if (used == 0 && ++spin > kSortSpin) prev += count_tile(kin, q--, shift, (uint32_t)t);
   }
   if (tile > 0) *mine = (tag_all << kShift) | (S)(prev + c);
   s_base[t] = first + prev - start;
@@ -239,7 +247,7 @@ int64_t sort_tiles(int64_t n) { return (n + kSortTile - 1) / kSortTile; }
 // counts: kCountWords words; look: sort_look_words(n) words.  ctx (may be
 // null): launch counting and timing.
 int sort_launches(art_ctx* ctx, cudaStream_t s, int sms, uint32_t* k0, uint32_t* v0, uint32_t* k1, uint32_t* v1,
-                  int64_t n, int key_bits, uint32_t* counts, uint32_t* look, unsigned long long* err) {
+                  int64_t n, int key_bits, uint32_t* counts, uint32_t* look) {
   const int64_t nt = sort_tiles(n);
   const int passes = key_bits / kRadixBits;
   cudaMemsetAsync(counts, 0, kCountWords * sizeof(uint32_t), s);
@@ -262,10 +270,10 @@ int sort_launches(art_ctx* ctx, cudaStream_t s, int sms, uint32_t* k0, uint32_t*
     if (ctx) prof_begin(ctx, "sort_pass");
     if (n < kSmallSort)
       cudaLaunchKernelEx(&cfg, radix_pass_kernel<uint32_t>, (const uint32_t*)K[src], (const uint32_t*)V[src], K[src ^ 1],
-                         V[src ^ 1], n, pass, counts, look, err);
+                         V[src ^ 1], n, pass, counts, look);
     else
       cudaLaunchKernelEx(&cfg, radix_pass_kernel<unsigned long long>, (const uint32_t*)K[src], (const uint32_t*)V[src],
-                         K[src ^ 1], V[src ^ 1], n, pass, counts, reinterpret_cast<unsigned long long*>(look), err);
+                         K[src ^ 1], V[src ^ 1], n, pass, counts, reinterpret_cast<unsigned long long*>(look));
     if (ctx) prof_end(ctx);
   }
   if (ctx) ctx->launches += 1 + passes;
@@ -827,8 +835,7 @@ void launch_tile_sort_views(art_ctx* ctx, const ViewSet& vs, int64_t ntiles) {
 
 int launch_sort(art_ctx* ctx, uint32_t* k0, uint32_t* v0, uint32_t* k1, uint32_t* v1, int64_t n, int key_bits,
                 uint32_t* counts, uint32_t* look) {
-  return sort_launches(ctx, ctx->stream, ctx->num_sms, k0, v0, k1, v1, n, key_bits, counts, look,
-                       ctx->d_status + kStScanError);
+  return sort_launches(ctx, ctx->stream, ctx->num_sms, k0, v0, k1, v1, n, key_bits, counts, look);
 }
 
 // ------------------------------------------------ sort without allocation
@@ -945,7 +952,7 @@ extern "C" art_status art_sort_pairs_static(uint32_t* keys, uint32_t* vals, int6
   int sms = 0;
   if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return (cudaGetLastError(), ART_ERR_CUDA);
   const int src = sort_launches(nullptr, s, sms, keys, vals, sk, sv, n, key_bits, (uint32_t*)(b + kOffCounts),
-                                (uint32_t*)(b + kOffLook), nullptr);
+                                (uint32_t*)(b + kOffLook));
   if (cudaPeekAtLastError() != cudaSuccess) return (cudaGetLastError(), ART_ERR_CUDA);
   if (src == 1) {
     if (cudaMemcpyAsync(keys, sk, sizeof(uint32_t) * (size_t)n, cudaMemcpyDeviceToDevice, s) != cudaSuccess ||

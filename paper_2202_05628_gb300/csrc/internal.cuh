@@ -45,7 +45,7 @@ enum StatusWord {
   kStSortBig = 16,      // binning: buckets sorted by a whole block
   kStSortBigNext = 17,  // binning: such buckets taken beyond each block's first (work counter)
   kStScanTicket = 18,   // binning: blocks of the tile scan started (their order)
-  kStScanError = 19,    // binning, sort: look-backs that timed out waiting for a predecessor
+  kStScanError = 19,    // binning: tile-scan blocks that timed out waiting for a predecessor
   kStActiveGroups = 20, // binning: groups of four consecutive tiles with instances (listed in d_agroups)
   kStExactQ = 21,       // composite: tiles queued for the exact re-walk (a pixel's reorder buffer overflowed)
   kStGridCells = 22,    // lattice index: occupied cells of the last pose
