@@ -22,6 +22,7 @@ art_status fail(art_ctx* ctx, art_status st, const char* fmt, ...) {
 }
 
 art_status cuda_fail(art_ctx* ctx, cudaError_t e, const char* what) {
+  cudaGetLastError();  // (reported here: the next call's launch check does not find it again)
   return fail(ctx, e == cudaErrorMemoryAllocation ? ART_ERR_OOM : ART_ERR_CUDA, "%s: %s", what,
               cudaGetErrorString(e));
 }

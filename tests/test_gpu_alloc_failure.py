@@ -1,0 +1,58 @@
+"""A device allocation that fails inside a call: the call reports it, and the
+next calls neither use what is missing nor forget to allocate it again.  The
+library is linked with a cudaMalloc that fails when told to."""
+import numpy as np
+import pytest
+
+import variants
+
+pytestmark = pytest.mark.gpu
+OOM = 3
+
+FAILING_MALLOC = """
+#include <stddef.h>
+int __real_cudaMalloc(void** p, size_t n);
+static int left = -1;  /* allocations until the one that fails (negative: none) */
+void fail_after(int n) { left = n; }
+int pending(void) { return left >= 0; }
+int __wrap_cudaMalloc(void** p, size_t n) {
+  if (left >= 0 && left-- == 0) n = (size_t)1 << 60; /* more than any device has: cudaErrorMemoryAllocation */
+  return __real_cudaMalloc(p, n);
+}
+"""
+
+
+@pytest.fixture(scope="module")
+def lib(tmp_path_factory):
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    return variants.library(tmp_path_factory.mktemp("alloc") / "liballoc.so", wrap=["cudaMalloc"], source=FAILING_MALLOC)
+
+
+@pytest.fixture
+def art(lib, monkeypatch):
+    import paper_2202_05628_gb300 as art
+    monkeypatch.setattr(art, "_lib", lib)
+    yield art
+    lib.fail_after(-1)
+
+
+def _sorted(r, n, seed):
+    import torch
+    k = np.random.default_rng(seed).integers(0, 2 ** 32, n, dtype=np.uint64).astype(np.uint32)
+    kt, vt = torch.from_numpy(k.view(np.int32)).cuda(), torch.arange(n, dtype=torch.int32, device="cuda")
+    r.sort_pairs(kt, vt)
+    order = np.argsort(k, kind="stable")
+    np.testing.assert_array_equal(vt.cpu().numpy(), order)
+    np.testing.assert_array_equal(kt.cpu().numpy().view(np.uint32), k[order])
+
+
+def test_a_reported_failure_is_not_reported_again(art, lib):
+    r = art.Renderer()
+    lib.fail_after(0)
+    with pytest.raises(art.ArtemisError) as e:
+        _sorted(r, 5000, 0)
+    assert e.value.status == OOM
+    _sorted(r, 5000, 0)
+    r.close()
