@@ -1279,6 +1279,7 @@ art_status art_sort_pairs(art_ctx* ctx, uint32_t* keys, uint32_t* vals, int64_t 
   if (!is_device_ptr(keys) || !is_device_ptr(vals)) return fail(ctx, ART_ERR_INVALID_ARG, "keys/vals must be device memory");
   art_status st;
   if (n > ctx->sort_cap) {
+    ctx->sort_cap = 0;  // (until all of it is there: an allocation that fails leaves null arrays)
     if ((st = alloc(ctx, &ctx->d_sk, (size_t)n, "sort scratch keys")) != ART_OK) return st;
     if ((st = alloc(ctx, &ctx->d_sv, (size_t)n, "sort scratch values")) != ART_OK) return st;
     if ((st = alloc(ctx, &ctx->d_slook, sort_look_words(n), "sort look-back words")) != ART_OK) return st;

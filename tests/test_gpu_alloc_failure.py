@@ -38,6 +38,24 @@ def art(lib, monkeypatch):
     lib.fail_after(-1)
 
 
+def _each_failure(art, lib, call):
+    """call() with its k-th allocation failing, k = 0, 1, ..., until it makes
+    no more; yields after each failure, which has to be reported as such."""
+    for k in range(100):
+        lib.fail_after(k)
+        try:
+            call()
+        except art.ArtemisError as e:
+            assert e.status == OOM, e
+            lib.fail_after(-1)
+            yield k
+        else:
+            assert lib.pending(), "an allocation failed without an error"
+            lib.fail_after(-1)
+            assert k > 0, "the call allocates nothing"
+            return
+
+
 def _sorted(r, n, seed):
     import torch
     k = np.random.default_rng(seed).integers(0, 2 ** 32, n, dtype=np.uint64).astype(np.uint32)
@@ -55,4 +73,15 @@ def test_a_reported_failure_is_not_reported_again(art, lib):
         _sorted(r, 5000, 0)
     assert e.value.status == OOM
     _sorted(r, 5000, 0)
+    r.close()
+
+
+def test_sort_scratch(art, lib):
+    r = art.Renderer()
+    _sorted(r, 5000, 0)
+    n = 5000
+    for k in _each_failure(art, lib, lambda: _sorted(r, 20000, 1)):
+        _sorted(r, n, 2 + k)  # (as many pairs as there was room for before)
+        n -= 1000
+    _sorted(r, 20000, 9)
     r.close()
