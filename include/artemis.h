@@ -165,7 +165,8 @@ art_status art_render_feature_maps(art_ctx* ctx, int view, void* F_out, int F_dt
  *   coef    [n][(degree+1)^2][C] float, host or device; copied
  * Errors: ART_ERR_STATE before art_load_octree, ART_ERR_UNSUPPORTED for a
  * degree above 3; art_render_backward and the learned skip then return
- * ART_ERR_UNSUPPORTED.  A new art_load_octree returns to the plain features.
+ * ART_ERR_UNSUPPORTED.  A new art_load_octree returns to the plain features,
+ * and so does a load that fails with ART_ERR_OOM or ART_ERR_CUDA.
  */
 art_status art_load_sh_features(art_ctx* ctx, int degree, const float* coef);
 

@@ -874,6 +874,7 @@ art_status art_load_sh_features(art_ctx* ctx, int degree, const float* coef) {
   if (!coef) return fail(ctx, ART_ERR_INVALID_ARG, "coef is null");
   const size_t count = (size_t)ctx->n * (size_t)((degree + 1) * (degree + 1)) * (size_t)ctx->C;
   art_status st;
+  ctx->sh_degree = -1;  // (until the coefficients are there)
   if ((st = alloc(ctx, &ctx->d_sh, count, "SH coefficients")) != ART_OK) return st;
   if ((st = alloc(ctx, &ctx->d_sh_rot, 3 * (size_t)ctx->n, "SH rotations")) != ART_OK) return st;
   cudaError_t e = cudaMemcpyAsync(ctx->d_sh, coef, sizeof(float) * count, cudaMemcpyDefault, ctx->stream);

@@ -4,7 +4,9 @@ library is linked with a cudaMalloc that fails when told to."""
 import numpy as np
 import pytest
 
+import scenegen as sg
 import variants
+from helpers import render_maps, renderer, set_cam, set_pose
 
 pytestmark = pytest.mark.gpu
 OOM = 3
@@ -85,3 +87,31 @@ def test_sort_scratch(art, lib):
         n -= 1000
     _sorted(r, 20000, 9)
     r.close()
+
+
+def test_sh_coefficients(art, lib):
+    """After a load that fails, the plain features are in use."""
+    sc = sg.preset("mini")
+    oc = sc.octree
+    cam = sg.orbit_camera(sc.centroid, 64, 64, az_deg=40.0)
+    rng = np.random.default_rng(3)
+    coef = [rng.standard_normal((oc.n, (L + 1) ** 2, oc.C)).astype(np.float32) for L in (1, 2)]
+
+    def fresh(L):
+        r = renderer(sc)
+        set_cam(r, 0, cam)
+        set_pose(r, sg.random_pose(2))
+        if L:
+            r.load_sh_features(L, coef[L - 1])
+        return r, render_maps(r, 0, cam, oc.C)
+
+    r, _ = fresh(1)
+    plain, want = fresh(0), fresh(2)
+    for _ in _each_failure(art, lib, lambda: r.load_sh_features(2, coef[1])):
+        for a, b in zip(render_maps(r, 0, cam, oc.C), plain[1]):
+            np.testing.assert_array_equal(a, b)
+        r.load_sh_features(1, coef[0])
+    for a, b in zip(render_maps(r, 0, cam, oc.C), want[1]):
+        np.testing.assert_array_equal(a, b)
+    for x in (r, plain[0], want[0]):
+        x.close()
