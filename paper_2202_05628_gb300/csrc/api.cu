@@ -187,6 +187,21 @@ art_status launch_check(art_ctx* ctx, const char* what) {
   return ART_OK;
 }
 
+void free_layers(art_ctx* ctx) {
+  for (auto& L : ctx->layers) {
+    if (L.w32) cudaFree(L.w32);
+    if (L.b32) cudaFree(L.b32);
+    if (L.wbf) cudaFree(L.wbf);
+    if (L.wsub) cudaFree(L.wsub);
+    if (L.wtap) cudaFree(L.wtap);
+    if (L.wx) cudaFree(L.wx);
+    if (L.wxu) cudaFree(L.wxu);
+    if (L.w8) cudaFree(L.w8);
+    if (L.wscale) cudaFree(L.wscale);
+  }
+  ctx->layers.clear();
+}
+
 void free_all(art_ctx* ctx) {
   void* ptrs[] = {ctx->d_ijk, ctx->d_jidx, ctx->d_w, ctx->d_feat, ctx->d_sigma, ctx->d_skel, ctx->d_pose, ctx->d_G,
                   ctx->d_rec, ctx->d_geo, ctx->d_rect, ctx->d_q, ctx->d_cnt, ctx->d_keys,
@@ -200,17 +215,7 @@ void free_all(art_ctx* ctx) {
                   ctx->d_gkeys, ctx->d_gvals, ctx->d_pgroups, ctx->d_tclass};
   for (void* p : ptrs)
     if (p) cudaFree(p);
-  for (auto& L : ctx->layers) {
-    if (L.w32) cudaFree(L.w32);
-    if (L.b32) cudaFree(L.b32);
-    if (L.wbf) cudaFree(L.wbf);
-    if (L.wsub) cudaFree(L.wsub);
-    if (L.wtap) cudaFree(L.wtap);
-    if (L.wx) cudaFree(L.wx);
-    if (L.wxu) cudaFree(L.wxu);
-    if (L.w8) cudaFree(L.w8);
-    if (L.wscale) cudaFree(L.wscale);
-  }
+  free_layers(ctx);
   if (ctx->h_status) cudaFreeHost(ctx->h_status);
   for (auto& t : ctx->pending) {
     cudaEventDestroy(t.e0);
@@ -911,67 +916,16 @@ art_status art_render_depth(art_ctx* ctx, int view, float sigma_min, float* dept
   return ART_OK;
 }
 
-art_status art_load_shader(art_ctx* ctx, const art_net_desc* desc, const float* params, int64_t n_params,
-                           int compute_dtype) {
-  if (!ctx) return ART_ERR_INVALID_ARG;
-  if (!desc || !params) return fail(ctx, ART_ERR_INVALID_ARG, "null descriptor or params");
-  if (compute_dtype != ART_F32 && compute_dtype != ART_BF16 && compute_dtype != ART_FP8)
-    return fail(ctx, ART_ERR_UNSUPPORTED, "compute dtype %d not available", compute_dtype);
-  std::vector<int> shapes;  // cout, cin, k
-  const art_net_desc& d = *desc;
-  // (cout, cin, k) of a U-Net's layers in execution order: enc0 a/b, ...,
-  // bottleneck a/b, dec(levels-2) a/b, ..., dec0 a/b, 1x1 head
-  auto unet_shapes = [&](int cin, int levels, const int* ch, int cout) {
-    int prev = cin;
-    for (int l = 0; l < levels; ++l) {
-      shapes.insert(shapes.end(), {ch[l], prev, 3, ch[l], ch[l], 3});
-      prev = ch[l];
-    }
-    for (int l = levels - 2; l >= 0; --l) shapes.insert(shapes.end(), {ch[l], ch[l + 1] + ch[l], 3, ch[l], ch[l], 3});
-    shapes.insert(shapes.end(), {cout, ch[0], 1});
-  };
-  if (d.cin < 1 || d.cout < 1 || d.cin > 256 || d.cout > 256) return fail(ctx, ART_ERR_INVALID_ARG, "cin/cout range");
-  if (d.arch == ART_NET_TINY) {
-    int c = d.ch[0];
-    if (c < 1 || c > 256) return fail(ctx, ART_ERR_INVALID_ARG, "hidden width range");
-    shapes = {c, d.cin, 3, c, c, 3, d.cout, c, 3};
-  } else if (d.arch == ART_NET_UNET || d.arch == ART_NET_TWO_BRANCH) {
-    for (int k = 0; k < 4; ++k)
-      if (d.ch[k] < 1 || d.ch[k] > 512) return fail(ctx, ART_ERR_INVALID_ARG, "channel range");
-    if (d.arch == ART_NET_UNET) {
-      unet_shapes(d.cin, 4, d.ch, d.cout);
-    } else {
-      if (d.cout != 4) return fail(ctx, ART_ERR_INVALID_ARG, "two-branch network: cout must be 4 (RGB + alpha)");
-      if (compute_dtype == ART_FP8) return fail(ctx, ART_ERR_UNSUPPORTED, "two-branch network: F32 or BF16 only");
-      for (int k = 0; k < 2; ++k)
-        if (d.ach[k] < 1 || d.ach[k] > 512) return fail(ctx, ART_ERR_INVALID_ARG, "opacity channel range");
-      unet_shapes(d.cin, 4, d.ch, 3);  // appearance: F -> I_f
-      unet_shapes(4, 2, d.ach, 1);     // opacity: [A, I_f] -> alpha
-    }
-  } else {
-    return fail(ctx, ART_ERR_INVALID_ARG, "unknown arch %d", d.arch);
-  }
-  int nl = (int)shapes.size() / 3;
-  int64_t need = 0;
-  for (int l = 0; l < nl; ++l) need += (int64_t)shapes[3 * l] * shapes[3 * l + 2] * shapes[3 * l + 2] * shapes[3 * l + 1] + shapes[3 * l];
-  if (need != n_params)
-    return fail(ctx, ART_ERR_INVALID_ARG, "n_params=%lld, network needs %lld", (long long)n_params, (long long)need);
-  for (auto& L : ctx->layers) {
-    if (L.w32) cudaFree(L.w32);
-    if (L.b32) cudaFree(L.b32);
-    if (L.wbf) cudaFree(L.wbf);
-    if (L.wsub) cudaFree(L.wsub);
-    if (L.wtap) cudaFree(L.wtap);
-    if (L.wx) cudaFree(L.wx);
-    if (L.wxu) cudaFree(L.wxu);
-    if (L.w8) cudaFree(L.w8);
-    if (L.wscale) cudaFree(L.wscale);
-  }
-  ctx->layers.clear();
+// The layers of network d (shapes: their cout, cin, k in execution order) and
+// the forms of their weights that the kernels of compute_dtype read.
+static art_status make_layers(art_ctx* ctx, const art_net_desc& d, const std::vector<int>& shapes, const float* params,
+                              int compute_dtype) {
+  const int nl = (int)shapes.size() / 3;
   int64_t off = 0;
   art_status st = ART_OK;
   for (int l = 0; l < nl; ++l) {
-    ConvLayer L;
+    ctx->layers.emplace_back();
+    ConvLayer& L = ctx->layers.back();
     L.cout = shapes[3 * l];
     L.cin = shapes[3 * l + 1];
     L.k = shapes[3 * l + 2];
@@ -996,7 +950,6 @@ art_status art_load_shader(art_ctx* ctx, const art_net_desc* desc, const float* 
       if ((st = alloc(ctx, &L.wscale, (size_t)L.cout, "fp8 weight scales")) != ART_OK) break;
       launch_quantize_weights(ctx, L.w32, L.cout, L.k * L.k * L.cin, L.w8, L.wscale);
     }
-    ctx->layers.push_back(L);
   }
   if (st != ART_OK) return st;
   // level 0's decoder convolution (after the concatenation with the
@@ -1075,6 +1028,57 @@ art_status art_load_shader(art_ctx* ctx, const art_net_desc* desc, const float* 
     ctx->f8_calibrated = false;
   }
   return sync_check(ctx, "load_shader");
+}
+
+art_status art_load_shader(art_ctx* ctx, const art_net_desc* desc, const float* params, int64_t n_params,
+                           int compute_dtype) {
+  if (!ctx) return ART_ERR_INVALID_ARG;
+  if (!desc || !params) return fail(ctx, ART_ERR_INVALID_ARG, "null descriptor or params");
+  if (compute_dtype != ART_F32 && compute_dtype != ART_BF16 && compute_dtype != ART_FP8)
+    return fail(ctx, ART_ERR_UNSUPPORTED, "compute dtype %d not available", compute_dtype);
+  std::vector<int> shapes;  // cout, cin, k
+  const art_net_desc& d = *desc;
+  // (cout, cin, k) of a U-Net's layers in execution order: enc0 a/b, ...,
+  // bottleneck a/b, dec(levels-2) a/b, ..., dec0 a/b, 1x1 head
+  auto unet_shapes = [&](int cin, int levels, const int* ch, int cout) {
+    int prev = cin;
+    for (int l = 0; l < levels; ++l) {
+      shapes.insert(shapes.end(), {ch[l], prev, 3, ch[l], ch[l], 3});
+      prev = ch[l];
+    }
+    for (int l = levels - 2; l >= 0; --l) shapes.insert(shapes.end(), {ch[l], ch[l + 1] + ch[l], 3, ch[l], ch[l], 3});
+    shapes.insert(shapes.end(), {cout, ch[0], 1});
+  };
+  if (d.cin < 1 || d.cout < 1 || d.cin > 256 || d.cout > 256) return fail(ctx, ART_ERR_INVALID_ARG, "cin/cout range");
+  if (d.arch == ART_NET_TINY) {
+    int c = d.ch[0];
+    if (c < 1 || c > 256) return fail(ctx, ART_ERR_INVALID_ARG, "hidden width range");
+    shapes = {c, d.cin, 3, c, c, 3, d.cout, c, 3};
+  } else if (d.arch == ART_NET_UNET || d.arch == ART_NET_TWO_BRANCH) {
+    for (int k = 0; k < 4; ++k)
+      if (d.ch[k] < 1 || d.ch[k] > 512) return fail(ctx, ART_ERR_INVALID_ARG, "channel range");
+    if (d.arch == ART_NET_UNET) {
+      unet_shapes(d.cin, 4, d.ch, d.cout);
+    } else {
+      if (d.cout != 4) return fail(ctx, ART_ERR_INVALID_ARG, "two-branch network: cout must be 4 (RGB + alpha)");
+      if (compute_dtype == ART_FP8) return fail(ctx, ART_ERR_UNSUPPORTED, "two-branch network: F32 or BF16 only");
+      for (int k = 0; k < 2; ++k)
+        if (d.ach[k] < 1 || d.ach[k] > 512) return fail(ctx, ART_ERR_INVALID_ARG, "opacity channel range");
+      unet_shapes(d.cin, 4, d.ch, 3);  // appearance: F -> I_f
+      unet_shapes(4, 2, d.ach, 1);     // opacity: [A, I_f] -> alpha
+    }
+  } else {
+    return fail(ctx, ART_ERR_INVALID_ARG, "unknown arch %d", d.arch);
+  }
+  int nl = (int)shapes.size() / 3;
+  int64_t need = 0;
+  for (int l = 0; l < nl; ++l) need += (int64_t)shapes[3 * l] * shapes[3 * l + 2] * shapes[3 * l + 2] * shapes[3 * l + 1] + shapes[3 * l];
+  if (need != n_params)
+    return fail(ctx, ART_ERR_INVALID_ARG, "n_params=%lld, network needs %lld", (long long)n_params, (long long)need);
+  free_layers(ctx);
+  const art_status st = make_layers(ctx, d, shapes, params, compute_dtype);
+  if (st != ART_OK) free_layers(ctx);  // (part of a network is none)
+  return st;
 }
 
 namespace art {

@@ -9,7 +9,7 @@ import variants
 from helpers import render_maps, renderer, set_cam, set_pose
 
 pytestmark = pytest.mark.gpu
-OOM = 3
+OOM, STATE = 3, 5
 
 FAILING_MALLOC = """
 #include <stddef.h>
@@ -115,3 +115,38 @@ def test_sh_coefficients(art, lib):
         np.testing.assert_array_equal(a, b)
     for x in (r, plain[0], want[0]):
         x.close()
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16", "fp8"])
+def test_shading_network(art, lib, dtype):
+    """After a load that fails there is no network."""
+    import torch
+    H, W, C = 24, 40, 32
+    nets = [sg.unet_weights(k, cin=C) for k in (1, 2)]
+    fdt, F_dtype = (torch.float32, "f32") if dtype == "f32" else (torch.bfloat16, "bf16")
+    F = torch.from_numpy(np.random.default_rng(1).standard_normal((H, W, C)).astype(np.float32)).cuda().to(fdt)
+
+    def load(r, k):
+        r.load_shader(art.ART_NET_UNET, C, sg.UNET_CHANNELS, 4, art.flat_params(nets[k]), dtype)
+
+    def shade(r):
+        out = torch.empty((H, W, 4), device="cuda")
+        r.shade(0, F, out, F_dtype)
+        r.sync_status()
+        return out
+
+    def fresh(k):
+        r = art.Renderer()
+        set_cam(r, 0, sg.orbit_camera((0.0, 0.0, 0.0), W, H))
+        load(r, k)
+        return r
+
+    r, ref = fresh(0), fresh(1)
+    shade(r)
+    for _ in _each_failure(art, lib, lambda: load(r, 1)):
+        with pytest.raises(art.ArtemisError) as e:
+            shade(r)
+        assert e.value.status == STATE
+    assert torch.equal(shade(r), shade(ref))
+    r.close()
+    ref.close()
