@@ -46,6 +46,8 @@ static bool pageable(const void* p) {
   return at.type == cudaMemoryTypeUnregistered;
 }
 
+// (A buffer is freed before its larger one is made, so whatever names its size
+// is reset first: an allocation that fails leaves a null pointer.)
 art_status ensure(art_ctx* ctx, void** p, size_t* have, size_t need, const char* what) {
   if (*p && *have >= need) return ART_OK;
   if (*p) cudaFree(*p);
@@ -256,12 +258,14 @@ art_status ensure_bin_buffers(art_ctx* ctx, int64_t ntiles) {
   const bool new_cap = cap != ctx->inst_cap, more_tiles = ntiles > ctx->ranges_cap;
   art_status st;
   if (new_cap) {
+    ctx->inst_cap = 0;
     if ((st = alloc(ctx, &ctx->d_keys, (size_t)cap, "instance keys")) != ART_OK) return st;
     if ((st = alloc(ctx, &ctx->d_vals, (size_t)cap, "instance values")) != ART_OK) return st;
     if ((st = alloc(ctx, &ctx->d_sort_tmp, (size_t)cap, "bucket staging")) != ART_OK) return st;
     ctx->inst_cap = cap;
   }
   if (more_tiles) {
+    ctx->ranges_cap = 0;
     if ((st = alloc(ctx, &ctx->d_ranges, (size_t)ntiles, "tile ranges")) != ART_OK) return st;
     if ((st = alloc(ctx, &ctx->d_tcount, (size_t)ntiles, "tile counts")) != ART_OK) return st;
     // zero once: from then on every tile scan zeroes the counts it read
@@ -283,6 +287,7 @@ art_status ensure_bin_buffers(art_ctx* ctx, int64_t ntiles) {
 art_status ensure_skip_buffers(art_ctx* ctx, const ViewParams& v) {
   art_status st;
   if (ctx->hist_n_cap < ctx->n) {
+    ctx->hist_n_cap = 0;
     if ((st = alloc(ctx, &ctx->d_hbin, (size_t)ctx->n, "voxel depth bins")) != ART_OK) return st;
     if ((st = alloc(ctx, &ctx->d_htau, (size_t)ctx->n, "voxel optical-depth bounds")) != ART_OK) return st;
     ctx->hist_n_cap = ctx->n;
@@ -326,7 +331,7 @@ art_status ensure_split_buffers(art_ctx* ctx, size_t ntiles) {
   }
   if ((st = ensure(ctx, (void**)&ctx->d_xqueue, &ctx->d_xqueue_bytes, ntiles * 4, "exact re-walk queue")) != ART_OK)
     return st;
-  if (!ctx->d_xhit) {
+  if (!ctx->d_xhit || !ctx->d_xpos) {
     const size_t m = (size_t)kExactBlocks * 32 * kExactCap;
     if ((st = alloc(ctx, &ctx->d_xhit, m, "exact re-walk hit lists")) != ART_OK) return st;
     if ((st = alloc(ctx, &ctx->d_xpos, m, "exact re-walk list positions")) != ART_OK) return st;
@@ -426,6 +431,8 @@ art_status art_load_octree(art_ctx* ctx, int64_t n, int depth, const float origi
     return fail(ctx, ART_ERR_INVALID_ARG, "storage_dtype %d invalid", storage_dtype);
   art_status st;
   size_t un = (size_t)n;
+  ctx->n = 0;  // (until the octree is there)
+  ctx->posed = false;
   if ((st = alloc(ctx, &ctx->d_ijk, un, "ijk")) != ART_OK) return st;
   if ((st = alloc(ctx, &ctx->d_jidx, un, "joint idx")) != ART_OK) return st;
   if ((st = alloc(ctx, &ctx->d_w, un, "weights")) != ART_OK) return st;
@@ -443,38 +450,39 @@ art_status art_load_octree(art_ctx* ctx, int64_t n, int depth, const float origi
   // staging for u16 ijk and FP32 features to convert
   uint16_t* t_ijk = nullptr;
   float* t_feat = nullptr;
-  if ((st = alloc(ctx, &t_ijk, 3 * un, "ijk staging")) != ART_OK) return st;
-  if ((st = copy_in(ctx, t_ijk, ijk, 3 * un * sizeof(uint16_t), "copy ijk")) != ART_OK) return st;
-  unsigned grid = (unsigned)((n + 255) / 256);
-  pack_ijk_kernel<<<grid, 256, 0, ctx->stream>>>(n, t_ijk, ctx->d_ijk);
-  if ((st = copy_in(ctx, ctx->d_jidx, joint_idx, un * 4, "copy joint idx")) != ART_OK) return st;
-  if ((st = copy_in(ctx, ctx->d_w, weights, un * 16, "copy weights")) != ART_OK) return st;
-  if ((st = copy_in(ctx, ctx->d_sigma, density, un * 4, "copy density")) != ART_OK) return st;
-  if (storage_dtype == ART_F32) {
-    if ((st = copy_in(ctx, ctx->d_feat, features, fbytes, "copy features")) != ART_OK) return st;
-  } else {
-    if ((st = alloc(ctx, &t_feat, un * C, "feature staging")) != ART_OK) return st;
-    if ((st = copy_in(ctx, t_feat, features, un * C * 4, "copy features")) != ART_OK) return st;
-    int64_t m = n * C;
-    unsigned g2 = (unsigned)((m + 255) / 256);
-    if (storage_dtype == ART_BF16)
-      convert_kernel<__nv_bfloat16><<<g2, 256, 0, ctx->stream>>>(m, t_feat, (__nv_bfloat16*)ctx->d_feat);
-    else
-      convert_kernel<__half><<<g2, 256, 0, ctx->stream>>>(m, t_feat, (__half*)ctx->d_feat);
-  }
-  // validate coordinates
-  cudaMemsetAsync(ctx->d_status + 7, 0, sizeof(unsigned long long), ctx->stream);
-  check_octree_kernel<<<grid, 256, 0, ctx->stream>>>(n, ctx->d_ijk, ctx->d_jidx, depth, ctx->d_status + 7);
-  cudaMemcpyAsync(ctx->h_status + 7, ctx->d_status + 7, sizeof(unsigned long long), cudaMemcpyDeviceToHost,
-                  ctx->stream);
-  st = sync_check(ctx, "load_octree");
-  cudaFree(t_ijk);
+  auto fill = [&]() -> art_status {
+    if ((st = alloc(ctx, &t_ijk, 3 * un, "ijk staging")) != ART_OK) return st;
+    if ((st = copy_in(ctx, t_ijk, ijk, 3 * un * sizeof(uint16_t), "copy ijk")) != ART_OK) return st;
+    unsigned grid = (unsigned)((n + 255) / 256);
+    pack_ijk_kernel<<<grid, 256, 0, ctx->stream>>>(n, t_ijk, ctx->d_ijk);
+    if ((st = copy_in(ctx, ctx->d_jidx, joint_idx, un * 4, "copy joint idx")) != ART_OK) return st;
+    if ((st = copy_in(ctx, ctx->d_w, weights, un * 16, "copy weights")) != ART_OK) return st;
+    if ((st = copy_in(ctx, ctx->d_sigma, density, un * 4, "copy density")) != ART_OK) return st;
+    if (storage_dtype == ART_F32) {
+      if ((st = copy_in(ctx, ctx->d_feat, features, fbytes, "copy features")) != ART_OK) return st;
+    } else {
+      if ((st = alloc(ctx, &t_feat, un * C, "feature staging")) != ART_OK) return st;
+      if ((st = copy_in(ctx, t_feat, features, un * C * 4, "copy features")) != ART_OK) return st;
+      int64_t m = n * C;
+      unsigned g2 = (unsigned)((m + 255) / 256);
+      if (storage_dtype == ART_BF16)
+        convert_kernel<__nv_bfloat16><<<g2, 256, 0, ctx->stream>>>(m, t_feat, (__nv_bfloat16*)ctx->d_feat);
+      else
+        convert_kernel<__half><<<g2, 256, 0, ctx->stream>>>(m, t_feat, (__half*)ctx->d_feat);
+    }
+    // validate coordinates
+    cudaMemsetAsync(ctx->d_status + 7, 0, sizeof(unsigned long long), ctx->stream);
+    check_octree_kernel<<<grid, 256, 0, ctx->stream>>>(n, ctx->d_ijk, ctx->d_jidx, depth, ctx->d_status + 7);
+    cudaMemcpyAsync(ctx->h_status + 7, ctx->d_status + 7, sizeof(unsigned long long), cudaMemcpyDeviceToHost,
+                    ctx->stream);
+    return sync_check(ctx, "load_octree");
+  };
+  st = fill();
+  if (t_ijk) cudaFree(t_ijk);
   if (t_feat) cudaFree(t_feat);
   if (st != ART_OK) return st;
-  if (ctx->h_status[7] != 0) {
-    ctx->n = 0;
+  if (ctx->h_status[7] != 0)
     return fail(ctx, ART_ERR_INVALID_ARG, "%llu voxels have ijk >= 2^depth", ctx->h_status[7]);
-  }
   ctx->n = n;
   ctx->depth = depth;
   for (int a = 0; a < 3; ++a) ctx->origin[a] = origin[a];
@@ -482,7 +490,6 @@ art_status art_load_octree(art_ctx* ctx, int64_t n, int depth, const float origi
   ctx->h = (float)((double)extent / (double)(1 << depth));
   ctx->C = C;
   ctx->feat_dtype = storage_dtype;
-  ctx->posed = false;
   ctx->jidx_ok = false;
   ctx->inst_cap = 0;  // force re-sizing of binning buffers
   return ART_OK;
@@ -501,6 +508,8 @@ art_status art_load_skeleton(art_ctx* ctx, int J, const int32_t* parent, const f
   for (int j = 1; j < J; ++j)
     if (par[j] < 0 || par[j] >= j) return fail(ctx, ART_ERR_INVALID_ARG, "parent[%d]=%d must be in [0, %d)", j, par[j], j);
   art_status st;
+  ctx->J = 0;  // (until the skeleton is there)
+  ctx->posed = false;
   if ((st = alloc(ctx, &ctx->d_skel, (size_t)5 * J, "skeleton")) != ART_OK) return st;
   if ((st = alloc(ctx, &ctx->d_pose, (size_t)3 * J + 6, "pose")) != ART_OK) return st;
   if ((st = alloc(ctx, &ctx->d_G, (size_t)12 * J, "joint transforms")) != ART_OK) return st;
@@ -519,7 +528,6 @@ art_status art_load_skeleton(art_ctx* ctx, int J, const int32_t* parent, const f
   ctx->J = J;
   memcpy(ctx->parent, par, sizeof(int32_t) * J);
   memcpy(ctx->rest, rest, sizeof(float) * 3 * J);
-  ctx->posed = false;
   ctx->jidx_ok = false;
   return ART_OK;
 }
@@ -589,10 +597,12 @@ art_status art_set_pose(art_ctx* ctx, const float* axis_angle, const float R[3],
       return fail(ctx, ART_ERR_INVALID_ARG, "%llu voxels reference joints >= J=%d", ctx->h_status[7], J);
     ctx->jidx_ok = true;
   }
+  ctx->posed = false;  // (until the pose is complete)
   launch_fk(ctx, by_arg ? &arg : nullptr);  // (zeroes the pose's counters, kStDegenerate and kStRmax)
   launch_lbs(ctx);
   if (ctx->cfg.index == ART_INDEX_GRID) {
     if (ctx->grid_slots < 2 * ctx->n) {
+      ctx->grid_slots = 0;
       int64_t slots = 1024;
       while (slots < 2 * ctx->n) slots <<= 1;
       if ((st = alloc(ctx, &ctx->d_gkeys, (size_t)slots, "lattice index keys")) != ART_OK) return st;
@@ -803,6 +813,7 @@ art_status art_render_views(art_ctx* ctx, int nv, const int* views, void* const*
   if ((st = ensure_split_buffers(ctx, (size_t)total)) != ART_OK) return st;
   const int64_t need = (int64_t)nv * ctx->n;
   if (ctx->views_cap < need) {
+    ctx->views_cap = 0;
     if ((st = alloc(ctx, &ctx->d_rect_v, (size_t)need, "batch voxel rects")) != ART_OK) return st;
     if ((st = alloc(ctx, &ctx->d_q_v, (size_t)need, "batch depth keys")) != ART_OK) return st;
     if ((st = alloc(ctx, &ctx->d_cnt_v, (size_t)need, "batch tile counts")) != ART_OK) return st;
@@ -1284,7 +1295,7 @@ art_status art_sort_pairs(art_ctx* ctx, uint32_t* keys, uint32_t* vals, int64_t 
   if (!is_device_ptr(keys) || !is_device_ptr(vals)) return fail(ctx, ART_ERR_INVALID_ARG, "keys/vals must be device memory");
   art_status st;
   if (n > ctx->sort_cap) {
-    ctx->sort_cap = 0;  // (until all of it is there: an allocation that fails leaves null arrays)
+    ctx->sort_cap = 0;
     if ((st = alloc(ctx, &ctx->d_sk, (size_t)n, "sort scratch keys")) != ART_OK) return st;
     if ((st = alloc(ctx, &ctx->d_sv, (size_t)n, "sort scratch values")) != ART_OK) return st;
     if ((st = alloc(ctx, &ctx->d_slook, sort_look_words(n), "sort look-back words")) != ART_OK) return st;
@@ -1346,6 +1357,7 @@ art_status art_render_backward(art_ctx* ctx, int view, const float* F, const flo
   if (st != ART_OK) return st;
   if ((st = ensure_split_buffers(ctx, (size_t)v.tiles_x * v.tiles_y)) != ART_OK) return st;
   if (ctx->gN_cap < ctx->n) {
+    ctx->gN_cap = 0;
     if ((st = alloc(ctx, &ctx->d_gN, (size_t)ctx->n * 12, "geometry gradient")) != ART_OK) return st;
     ctx->gN_cap = ctx->n;
   }

@@ -325,17 +325,14 @@ art_status load_proposal(art_ctx* ctx, const float* params) {
     float* bdst = l < 4 ? &f32[64 * kPoseIn + 64 * l] : &f32[64 * kPoseIn + 256];
     for (int n = 0; n < N; ++n) bdst[n] = P[off[l][1] + n];
   }
-  art_status st;
-  if (!ctx->d_prop_img) {
-    if (cudaMalloc(&ctx->d_prop_img, kImgBytes) != cudaSuccess || cudaMalloc(&ctx->d_prop_f32, 4 * kF32Words) != cudaSuccess ||
-        cudaMalloc(&ctx->d_pose_bias, 4 * 64) != cudaSuccess)
-      return fail(ctx, ART_ERR_OOM, "proposal buffers");
-  }
+  if ((!ctx->d_prop_img && (e = cudaMalloc(&ctx->d_prop_img, kImgBytes)) != cudaSuccess) ||
+      (!ctx->d_prop_f32 && (e = cudaMalloc(&ctx->d_prop_f32, 4 * kF32Words)) != cudaSuccess) ||
+      (!ctx->d_pose_bias && (e = cudaMalloc(&ctx->d_pose_bias, 4 * 64)) != cudaSuccess))
+    return cuda_fail(ctx, e, "proposal buffers");
   if ((e = cudaMemcpy(ctx->d_prop_img, img.data(), kImgBytes, cudaMemcpyHostToDevice)) != cudaSuccess ||
       (e = cudaMemcpy(ctx->d_prop_f32, f32.data(), 4 * kF32Words, cudaMemcpyHostToDevice)) != cudaSuccess)
     return cuda_fail(ctx, e, "upload proposal");
   ctx->prop_loaded = true;
-  (void)st;
   return ART_OK;
 }
 
