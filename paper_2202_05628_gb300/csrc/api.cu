@@ -293,11 +293,11 @@ art_status ensure_skip_buffers(art_ctx* ctx, const ViewParams& v) {
     ctx->hist_n_cap = ctx->n;
   }
   const size_t ntiles = (size_t)v.tiles_x * v.tiles_y;
-  const float* thist_was = ctx->d_thist;
+  const size_t thist_was = ctx->d_thist_bytes;  // (a new buffer may get the old one's address)
   if ((st = ensure(ctx, (void**)&ctx->d_thist, &ctx->d_thist_bytes, ntiles * kPropBins * 4, "tile histogram")) != ART_OK)
     return st;
   // zeroed once; the tile scan zeroes the rows of the tiles it gives instances
-  if (ctx->d_thist != thist_was) cudaMemsetAsync(ctx->d_thist, 0, ctx->d_thist_bytes, ctx->stream);
+  if (ctx->d_thist_bytes != thist_was) cudaMemsetAsync(ctx->d_thist, 0, ctx->d_thist_bytes, ctx->stream);
   if ((st = ensure(ctx, (void**)&ctx->d_fbq, &ctx->d_fbq_bytes, ntiles * 4, "fallback queue")) != ART_OK) return st;
   if ((st = ensure(ctx, (void**)&ctx->d_bins, &ctx->d_bins_bytes, (size_t)v.W * v.H * 2, "proposal bins")) != ART_OK)
     return st;
@@ -322,10 +322,10 @@ art_status ensure_split_buffers(art_ctx* ctx, size_t ntiles) {
   if ((st = ensure(ctx, (void**)&ctx->d_fbq, &ctx->d_fbq_bytes, ntiles * 4, "fallback queue")) != ART_OK) return st;
   if ((st = ensure(ctx, (void**)&ctx->d_fbq2, &ctx->d_fbq2_bytes, ntiles * 4, "coarse-check failures")) != ART_OK)
     return st;
-  const uint32_t* xflag_was = ctx->d_xflag;
+  const size_t xflag_was = ctx->d_xflag_bytes;  // (a new buffer may get the old one's address)
   if ((st = ensure(ctx, (void**)&ctx->d_xflag, &ctx->d_xflag_bytes, ntiles * 4, "exact re-walk flags")) != ART_OK)
     return st;
-  if (ctx->d_xflag != xflag_was) {  // stamps start over on a new array
+  if (ctx->d_xflag_bytes != xflag_was) {  // stamps start over on a new array
     cudaMemsetAsync(ctx->d_xflag, 0, ctx->d_xflag_bytes, ctx->stream);
     ctx->xstamp = 0;
   }
