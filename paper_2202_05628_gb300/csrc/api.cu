@@ -997,14 +997,7 @@ static art_status make_layers(art_ctx* ctx, const art_net_desc& d, const std::ve
   // the FP32 network on the tensor cores: every 3x3 layer's weight parts,
   // where the widths are ones its kernel takes (else the CUDA-core kernels)
   if (st == ART_OK && compute_dtype == ART_F32) {
-    auto unet_ok = [&](int levels, const int* ch) {
-      bool ok = ch[0] == 32;  // (the 1x1 head is fused into a 32-channel layer)
-      for (int l = 0; l < levels; ++l) ok = ok && (ch[l] == 32 || ch[l] % 64 == 0);
-      return ok;
-    };
-    bool ok = d.arch == ART_NET_TINY ? d.ch[0] == 32 && d.cout <= 32 : unet_ok(4, d.ch) && d.cout <= 4;
-    if (d.arch == ART_NET_TWO_BRANCH) ok = ok && unet_ok(2, d.ach);
-    for (const ConvLayer& L : ctx->layers) ok = ok && (L.k == 1 || x3_layer_ok(L));
+    const bool ok = x3_net_ok(d);
     auto parts = [&](int li, int cu) -> art_status {  // cu: channels of the upsampled tensor, first in the concatenation
       ConvLayer& L = ctx->layers[li];
       art_status s2 = alloc(ctx, &L.wx, x3_weight_elems(L.cout, L.cin - cu, 9), "weight parts");

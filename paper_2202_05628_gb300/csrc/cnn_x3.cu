@@ -805,8 +805,14 @@ art_status launch_n(art_ctx* ctx, const X3Conv& c) {
 int x3_cin_pad(int c) { return (c + kKC - 1) / kKC * kKC; }
 int x3_cout_pad(int c) { return c <= 32 ? 32 : c; }
 
-bool x3_layer_ok(const ConvLayer& L) {
-  return L.k == 3 && L.cout <= kMaxCout && (L.cout <= 32 || L.cout % 64 == 0) && tensor_map_encoder() != nullptr;
+bool x3_net_ok(const art_net_desc& d) {
+  if (tensor_map_encoder() == nullptr) return false;
+  auto width_ok = [](int c) { return c <= kMaxCout && (c == 32 || c % 64 == 0); };
+  if (d.arch == ART_NET_TINY) return d.ch[0] == 32 && d.cout <= 32;
+  bool ok = d.ch[0] == 32 && d.cout <= 4;
+  for (int c : d.ch) ok = ok && width_ok(c);
+  if (d.arch == ART_NET_TWO_BRANCH) ok = ok && d.ach[0] == 32 && width_ok(d.ach[1]);
+  return ok;
 }
 
 size_t x3_weight_elems(int cout, int cin, int taps) { return (size_t)taps * 3 * x3_cout_pad(cout) * x3_cin_pad(cin); }

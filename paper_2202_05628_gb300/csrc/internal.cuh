@@ -510,7 +510,10 @@ struct X3Conv {
   const ConvLayer* head = nullptr;
   int out_ld = 0, out_off = 0;
 };
-bool x3_layer_ok(const ConvLayer& L);
+// Networks whose every 3x3 layer it takes: 32 channels at the first level (the
+// 1x1 head is fused into a 32-channel layer of at most four outputs), 32 or a
+// multiple of 64 at the others.
+bool x3_net_ok(const art_net_desc& d);
 int x3_cin_pad(int c);   // stored channels of a parts tensor
 int x3_cout_pad(int c);
 size_t x3_weight_elems(int cout, int cin, int taps);
