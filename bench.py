@@ -311,7 +311,7 @@ def composite_roofline(kt, stats, peaks, form, C, frames):
 
 def unet_flops(H, W, cin=32, ch=(32, 64, 128, 256), subpixel=False):
     """FLOPs of the 4-level U-Net on an H x W map.  subpixel: as the BF16
-    tensor-core network executes it, each decoder block's first convolution
+    and FP32 tensor-core networks execute it, each decoder block's first convolution
     over [up2(d) | e] in its sub-pixel form (the upsampled part through 4
     taps per output pixel instead of 9)."""
     import scenegen as sg

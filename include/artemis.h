@@ -114,6 +114,9 @@ art_status art_load_skeleton(art_ctx* ctx, int J, const int32_t* parent, const f
  * A_i = sum_k w_ik G_{j_ik}, its inverse, and its warped bounding data.
  *   axis_angle  [J][3] joint rotations r (axis-angle, radians)
  *   R[3], T[3]  global rotation (axis-angle) and translation (metres)
+ * Pageable arrays are read during the call, pinned and device arrays by the
+ * stream; under stream capture all are read when the graph is replayed, and
+ * have to live as long as it does.
  * Voxels whose blended 3x3 part has det < 1e-3 are dropped from rendering and
  * counted in art_stats.degenerate.
  */
@@ -242,8 +245,9 @@ typedef struct {
  *       with art_shade_with_opacity (it needs A); F32 or BF16 only.
  * params: float array, for every layer in execution order its weights
  *   [Cout][k][k][Cin] followed by its bias [Cout]; n_params must match.
- * compute_dtype: ART_F32 (FP32: on the tensor cores as exact three-part BF16
- *   products where the widths allow, else on CUDA cores), ART_BF16 (tensor cores, BF16
+ * compute_dtype: ART_F32 (FP32: on the tensor cores where the widths allow, each
+ *   value as three BF16 parts whose sum it is exactly from 2^-110 up, else on
+ *   CUDA cores), ART_BF16 (tensor cores, BF16
  *   operands, FP32 accumulation) or ART_FP8 (U-Net only: E4M3 operands,
  *   FP32 accumulation, per-output-channel weight scales max|w_co| / 448 and
  *   per-tensor activation scales; each art_shade quantises with the scales
@@ -383,7 +387,10 @@ typedef struct {
                               (0 = default 1e-3); a tile above it is traversed in full */
   int margin;              /* learned skip: bins added on both sides of the predicted interval (default 0) */
   int segment;             /* composite: a tile's list is walked in segments of about this many entries by
-                              separate warps and merged front to back (0 = default 256; >= 32) */
+                              separate warps and merged front to back (0 = default 256; >= 32).  At the
+                              default, asked for by 0 or by 256, art_render_backward cuts shorter ones
+                              (down to 64) where a view has too few for the GPU; other lengths hold
+                              for it as given */
   int index;               /* ART_INDEX_BOXES (default): every warped voxel is its exact parallelepiped;
                               ART_INDEX_GRID: the paper's per-frame index (Sec. 3.1 "Dynamic Volume
                               Rendering"): each warped centre is snapped to the cell of the leaf lattice

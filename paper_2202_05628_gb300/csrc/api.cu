@@ -543,8 +543,8 @@ static art_status ensure_side(art_ctx* ctx) {
   return ART_OK;
 }
 
-// The proposal's per-pose bias runs on the side stream beside FK and LBS;
-// work on the main stream that reads the bias or the proposal's weights
+// The proposal's per-pose bias runs on the side stream after FK and LBS, beside
+// the projection and binning that follow; work on the main stream that reads the bias or the proposal's weights
 // waits for it first (pose_bias_join).
 static art_status pose_bias_beside(art_ctx* ctx) {
   art_status st = ensure_side(ctx);

@@ -33,8 +33,9 @@
 // pixels (TMA fills zeros), which is exact: an upsampled pixel outside the
 // image maps to a low-resolution one outside it.
 //
-// Bound by shared memory (an MMA of 32 or 64 columns reads its operands at 128
-// bytes a cycle; ~74 cycles per MMA against 43) at 27 % tensor-pipe time.
+// An MMA takes ~74 cycles here at 27 % tensor-pipe time; reading its operands
+// (32 or 64 columns) from shared memory at 128 bytes a cycle accounts for 43,
+// the boxes and the staged stores for part of the rest, some has no known cause.
 // 1024x1024, 96 -> 32 channels: 77 us, 57 without divisions on the issuing
 // threads, 55 with the skip blocks kept once (six stages instead of four).
 #include <cuda.h>

@@ -793,8 +793,9 @@ __global__ void __launch_bounds__(kRowThreads, (RowCfg<N, KCB, F8>::kMinCtas))
     // two warps per TMEM lane quarter, each two of the unit's four rows: a row
     // takes a warp ~1700 cycles (its loads, transposes and stores one after the
     // other), four of them longer than the unit's MMAs.  (1920x1080, 64 -> 64
-    // channels 52 -> 44 us; the 32-channel layers, 54-60 us, are bound by shared
-    // memory: operand reads, boxes and staging are ~37 us of it)
+    // channels 52 -> 44 us; of the 32-channel layers' 54-60 us the shared-memory
+    // time of operand reads, boxes and staging, one after the other, accounts for
+    // ~37, the rest has no known cause)
     const int qd = warp & 3, r0 = ((warp - 2) >> 2) * (kRows / 2);
     const int m = qd * 32 + lane;
     const uint32_t tq = tmem_base + ((uint32_t)(qd * 32) << 16);  // this warp's lane quarter

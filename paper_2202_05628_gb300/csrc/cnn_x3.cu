@@ -1,8 +1,9 @@
 // The FP32 shading network's 3x3 convolutions on the tensor cores (arXiv
 // 2202.05628, Sec. 3.1 "Neural Shading"), at FP32 precision.
 //
-// An FP32 value is exactly the sum of three BF16 parts (x = x1 + x2 + x3,
-// each part the rounding of what the earlier ones leave), so a product is
+// An FP32 value is the sum of three BF16 parts (x = x1 + x2 + x3, each part
+// the rounding of what the earlier ones leave; exactly from 2^-110 up, below
+// that bits under 2^-133, the smallest BF16 value, are lost), so a product is
 //   w x = w1 x1 + (w1 x2 + w2 x1) + (w2 x2 + w1 x3 + w3 x1) + O(2^-24 |w x|),
 // six BF16 products of which each is exact in FP32.  tcgen05.mma truncates
 // its FP32 sums, so two things keep the error below that of a chain of FP32
@@ -34,9 +35,10 @@
 // registers, its drains outlast the other row's MMAs, and small images have
 // half as many units.
 //
-// Bounds: shared-memory bandwidth (operand reads are ~125 B a clock at these N,
-// the TMA boxes and the staged stores come on top): 49-61 % tensor-pipe time for
-// N = 64; for N = 32 (36-42 %) also the epilogue between its short units.
+// Bounds: at these N operand reads alone take ~125 B of shared memory a clock of
+// MMA time, and the TMA boxes and the staged stores come on top: 49-61 %
+// tensor-pipe time for N = 64; for N = 32 (36-42 %) also the epilogue between
+// its short units.
 // Measured: FP32 frame of 1M voxels at 1024x1024 10.21 ms with the CUDA-core
 // kernels (36 TFLOP/s) -> 1.74 ms; the U-Net at 424x248 1720 -> 351 us.
 //
@@ -116,7 +118,7 @@ __device__ __forceinline__ float part_sum(const __nv_bfloat16* p, int plane) {
   return (__bfloat162float(p[0]) + __bfloat162float(p[plane])) + __bfloat162float(p[2 * plane]);
 }
 
-// The parts of x (x = sum, exactly): rounded to nearest, the first toward
+// The parts of x (x = sum, exactly from 2^-110 up): rounded to nearest, the first toward
 // zero where rounding would overflow; an infinity or NaN is its own first part.
 __device__ __forceinline__ void split3(float x, __nv_bfloat16& a, __nv_bfloat16& b, __nv_bfloat16& c) {
   a = __float2bfloat16_rn(x);
@@ -386,7 +388,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   uint64_t* acce = accf + 2;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acce + 2);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
-  // the layer's biases (read per unit: from global memory their latencies cost ~27 us a unit at N = 128)
+  // the layer's biases (every unit reads them: from global memory each would wait for them)
   float* s_bias = reinterpret_cast<float*>((reinterpret_cast<uintptr_t>(tmem_slot + 4) + 15) & ~(uintptr_t)15);
   float* s_head = s_bias + kMaxCout;  // [4][32] weights, [4] biases
 
